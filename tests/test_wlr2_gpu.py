@@ -49,6 +49,22 @@ def test_wlr2_matches_oracle(W, H, F, r, T, rgb, b, groups, monkeypatch):
     assert err.max() <= TOL
 
 
+@pytest.mark.parametrize("W,H,F,r,T", [
+    (1, 1, 1, 1, 1),       # one pixel, one neighbour in the image
+    (16, 1, 1, 3, 1),      # exactly one 16 x 1 pixel group
+    (17, 2, 2, 2, 2),      # one pixel past it
+    (8, 4, 1, 3, 1),       # 8 x 2 pixel groups
+    (9, 5, 1, 3, 1),       # and their remainders
+    (12, 9, 3, 5, 3),      # more than 128 neighbour pairs: flushed partial sums
+    (20, 17, 2, 12, 2),    # a window larger than the image, several tables per frame
+])
+def test_wlr2_pixel_groups_and_partial_sums(W, H, F, r, T):
+    rad, feat = _inputs(W, H, F, True, seed=11)
+    g = _gpu(rad, feat, (0.8, 1.2, 1.0, 1.5, 0.9, 1.1, 1.0), radius=r, frames=T)
+    o = O.wlr2(rad.numpy(), feat.numpy(), bandwidth=(0.8, 1.2, 1.0, 1.5, 0.9, 1.1, 1.0), radius=r, frames=T)
+    assert np.abs(g - o).max() <= TOL
+
+
 def test_wlr2_image_smaller_than_window():
     rad, feat = _inputs(5, 3, 2, True, seed=7)
     g = _gpu(rad, feat, radius=3, frames=2)
