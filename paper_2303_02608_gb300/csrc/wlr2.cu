@@ -31,8 +31,9 @@
 // another's instructions: 2.9 of 7 stalls per issue were fetches.  Nine warps
 // and nine cyclic variables take 88 sums, but load the four schedulers
 // unevenly, and only 96 registers fit.)  The representatives are products of a
-// row term (w v_0 v_k, k <= 3, and the lower degrees) and one of 16 column
-// pairs v_c v_d, chosen so that the pairs reach every orbit.
+// row term (w v_0 v_k, and the lower degrees) and one of 16 column pairs v_c
+// v_d, chosen so that the pairs reach every orbit and that the rows that a
+// column needs come in twos: 98 of the 100 sums are updated by 49 packed FMAs.
 //
 // Layout of the work: a CTA of 256 threads takes 16 pixels of one frame (16 x 1
 // or 8 x 2).  A lane is a (pixel, half) pair: the two halves of a warp take
@@ -43,12 +44,13 @@
 // memory, so long windows do not lengthen the FP32 sums.
 //
 // The solve keeps the matrix in shared memory, [element][pixel]: a lane works
-// on its own pixel, so every step of the blocked Cholesky (8 block columns of
-// 7, left-looking, one tile per warp, its columns split over the halves) runs
-// all its lanes, and operands are read without bank conflicts.  Two CTAs per SM: one
+// on its own pixel, so every step of the blocked Cholesky (7 block columns of
+// 8, one tile per warp, its even and odd columns on the halves) runs all its
+// lanes, and operands are read without bank conflicts.  Two CTAs per SM: one
 // solves (latency-bound) while the other accumulates (FMA-bound).
 //
-// Measured at 512 x 512 x 16, 7 x 7 x 3 window: 55.7 ms, against 92.0 ms with the
+// Measured at 512 x 512 x 16, 7 x 7 x 3 window: 46.7 ms (55.7 with single FMAs,
+// blocks of 7 and a wholly left-looking order), against 92.0 ms with the
 // Gram accumulated as 36 7 x 7 register tiles (1764 sums per neighbour) and
 // factored in registers, 36 threads per pixel.
 #include <stdlib.h>
@@ -94,29 +96,32 @@ __host__ __device__ constexpr int pair_b(int q)
 
 // A sum in terms of the rotated variables x_0..x_7: row term times x_c x_d (c <=
 // d), x_c alone (d = -1), or the warp's own sum without any x (c = -1).
-// Row terms: factors x_0 x_k or x_0 or none, times a power of z, times w or w y.
+// Row terms: factors x_0 x_k or x_0 or none, times a power of z, times w or w y;
+// rows 2r and 2r + 1 are a pair.
 struct Row {
     signed char n, k, z, y;   // number of x factors; the second is x_k; power of z; times y
 };
 constexpr int kRows = 12;
-constexpr Row kRow[kRows] = {{2, 0, 0, 0}, {2, 1, 0, 0}, {2, 2, 0, 0}, {2, 3, 0, 0}, {1, 0, 0, 0}, {1, 0, 1, 0},
-                             {0, 0, 0, 0}, {0, 0, 1, 0}, {0, 0, 2, 0}, {0, 0, 3, 0}, {0, 0, 0, 1}, {0, 0, 1, 1}};
+constexpr Row kRow[kRows] = {{2, 0, 0, 0}, {2, 2, 0, 0}, {2, 1, 0, 0}, {2, 4, 0, 0}, {1, 0, 0, 0}, {1, 0, 1, 0},
+                             {0, 0, 0, 0}, {0, 0, 1, 0}, {0, 0, 2, 0}, {0, 0, 0, 1}, {0, 0, 3, 0}, {0, 0, 1, 1}};
 
 struct Sum {
     signed char row, c, d;
 };
 
 struct SumList {
-    Sum s[kSums];
+    Sum s[kSums];   // 2i and 2i + 1: a pair of rows times one column, but for the last two
     int n;
 };
 
-// Column pairs, found by a search over hitting sets: every orbit of degree 4
-// has a rotation {0, k, c, d} with k <= 3 and (c, d) among them, every orbit of
-// degree 3 one {0, c, d}, every orbit of degree 2 one (c, d).
+// Column pairs in the order of their use, found by a search: every orbit of
+// degree 4 has a rotation {0, k, c, d}, k in {0, 1, 2, 4}, with (c, d) among
+// them, every orbit of degree 3 one {0, c, d}, every orbit of degree 2 one
+// (c, d); and taken in this order 42 of the 43 orbits of degree 4 fall into
+// whole row pairs.
 constexpr int kCols = 16;
-constexpr signed char kCol[kCols][2] = {{0, 0}, {0, 4}, {0, 5}, {0, 6}, {1, 1}, {1, 2}, {1, 6}, {3, 5},
-                                        {3, 7}, {4, 4}, {4, 6}, {4, 7}, {5, 5}, {5, 6}, {6, 6}, {7, 7}};
+constexpr signed char kCol[kCols][2] = {{7, 7}, {0, 6}, {1, 7}, {5, 5}, {1, 5}, {0, 7}, {0, 3}, {5, 6},
+                                        {0, 0}, {2, 6}, {6, 6}, {5, 7}, {3, 6}, {0, 4}, {1, 4}, {0, 5}};
 
 // The orbit of {v_0..v_(n-1)}: its smallest rotation, as a number.
 __host__ __device__ constexpr int orbit(const int (&v)[4], int n)
@@ -135,28 +140,46 @@ __host__ __device__ constexpr int orbit(const int (&v)[4], int n)
 __host__ __device__ constexpr SumList sum_list()
 {
     SumList l{};
-    int seen[kSums] = {}, n_seen = 0;
+    int seen[kSums] = {}, n_seen = 0;   // orbits (the codes of different degrees differ)
+    Sum last{};                         // the single sum of degree 4
+    auto is_new = [&](int key) {
+        for (int i = 0; i < n_seen; ++i)
+            if (seen[i] == key) return false;
+        return true;
+    };
     for (int q = 0; q < kCols; ++q) {
         const int c = kCol[q][0], d = kCol[q][1];
-        for (int row = 0; row <= 6; ++row) {
-            if (row == 5) continue;   // goes with row 4
-            const int four[4] = {0, row, c, d}, three[4] = {0, c, d, 0}, two[4] = {c, d, 0, 0};
-            const int key = row <= 3 ? orbit(four, 4) : row == 4 ? orbit(three, 3) : orbit(two, 2);
-            bool dup = false;
-            for (int i = 0; i < n_seen; ++i) dup |= seen[i] == key;   // (the codes of different degrees differ)
-            if (dup) continue;
-            seen[n_seen++] = key;
-            auto add = [&](int r) { l.s[l.n++] = Sum{(signed char)r, (signed char)c, (signed char)d}; };
-            add(row);
-            if (row == 4) add(5);
-            if (row == 6) {
-                add(7);
-                add(8);
-                add(10);
+        auto add = [&](int row, int cc, int dd) { l.s[l.n++] = Sum{(signed char)row, (signed char)cc, (signed char)dd}; };
+        for (int r = 0; r < 2; ++r) {
+            const int lo[4] = {0, kRow[2 * r].k, c, d}, hi[4] = {0, kRow[2 * r + 1].k, c, d};
+            const int kl = orbit(lo, 4), kh = orbit(hi, 4);
+            if (is_new(kl) && is_new(kh) && kl != kh) {
+                seen[n_seen++] = kl;
+                seen[n_seen++] = kh;
+                add(2 * r, c, d);
+                add(2 * r + 1, c, d);
             }
         }
+        for (int row = 0; row < 4; ++row) {
+            const int four[4] = {0, kRow[row].k, c, d}, key = orbit(four, 4);
+            if (is_new(key)) {
+                seen[n_seen++] = key;
+                last = Sum{(signed char)row, (signed char)c, (signed char)d};
+            }
+        }
+        const int three[4] = {0, c, d, 0}, two[4] = {c, d, 0, 0};
+        if (is_new(orbit(three, 3))) {
+            seen[n_seen++] = orbit(three, 3);
+            add(4, c, d);
+            add(5, c, d);
+        }
+        if (is_new(orbit(two, 2))) {
+            seen[n_seen++] = orbit(two, 2);
+            for (int row = 6; row < 10; ++row) add(row, c, d);
+        }
     }
-    for (int row = 6; row <= 11; ++row) l.s[l.n++] = Sum{(signed char)row, 0, -1};
+    for (int row = 6; row < 12; ++row) l.s[l.n++] = Sum{(signed char)row, 0, -1};
+    l.s[l.n++] = last;
     l.s[l.n++] = Sum{6, -1, -1};
     return l;
 }
@@ -173,21 +196,22 @@ __host__ __device__ constexpr int gram_row(int p, int q)
     return z + (q - p);
 }
 
-// First element of tile (I, J), I <= J, of the packed upper triangle: 7 x 7
-// tiles in row order, diagonal tiles packed to 28.
+// First element of tile (I, J), I <= J, of the packed upper triangle: 8 x 8
+// tiles in row order, diagonal tiles packed to 36.
+constexpr int kB = 8, kNB = kNA / kB, kDiag = kB * (kB + 1) / 2;
 __host__ __device__ constexpr int tile_base(int I, int J)
 {
-    return 28 * I + 49 * (7 * I - I * (I - 1) / 2) + (J > I ? 28 + 49 * (J - I - 1) : 0);
+    return kDiag * I + kB * kB * ((kNB - 1) * I - I * (I - 1) / 2) + (J > I ? kDiag + kB * kB * (J - I - 1) : 0);
 }
-static_assert(tile_base(7, 7) + 28 == kElems, "packed triangle");
+static_assert(tile_base(kNB - 1, kNB - 1) + kDiag == kElems, "packed triangle");
 
-__host__ __device__ constexpr int diag_elem(int r, int c) { return r * 7 - r * (r - 1) / 2 + (c - r); }
+__host__ __device__ constexpr int diag_elem(int r, int c) { return r * kB - r * (r - 1) / 2 + (c - r); }
 
 __host__ __device__ constexpr int elem(int i, int j)
 {
     const int lo = i < j ? i : j, hi = i < j ? j : i;
-    const int I = lo / 7, J = hi / 7;
-    return tile_base(I, J) + (I == J ? diag_elem(lo % 7, hi % 7) : (lo % 7) * 7 + hi % 7);
+    const int I = lo / kB, J = hi / kB;
+    return tile_base(I, J) + (I == J ? diag_elem(lo % kB, hi % kB) : (lo % kB) * kB + hi % kB);
 }
 
 // Places of the Gram (element numbers of the packed triangle) that sum i of
@@ -283,17 +307,24 @@ __global__ void __launch_bounds__(kTilePix) wlr2_pack_kernel(W2Params p)
 
 // One neighbour: x the rotated variables, own the warp's own term.
 template <int... I>
-__device__ __forceinline__ void add_sums(float (&acc)[kSums], float w, float wy, float z, float own,
+__device__ __forceinline__ void add_sums(float2 (&acc)[kSums / 2], float w, float wy, float z, float own,
                                          const float (&x)[8], std::integer_sequence<int, I...>)
 {
     const float wx = w * x[0], wz = w * z, wzz = wz * z;
-    const float row[kRows] = {wx * x[0], wx * x[1], wx * x[2], wx * x[3], wx, wz * x[0],
-                              w, wz, wzz, wzz * z, wy, wy * z};
-    auto term = [&](auto idx, float& a) {
-        constexpr Sum m = kList.s[decltype(idx)::value];
-        if constexpr (m.c < 0) a += own;
-        else if constexpr (m.d < 0) a = fmaf(row[m.row], x[m.c], a);
-        else a = fmaf(row[m.row], x[m.c] * x[m.d], a);
+    const float2 row[kRows / 2] = {make_float2(wx * x[0], wx * x[2]), make_float2(wx * x[1], wx * x[4]),
+                                   make_float2(wx, wz * x[0]),        make_float2(w, wz),
+                                   make_float2(wzz, wy),              make_float2(wzz * z, wy * z)};
+    auto term = [&](auto idx, float2& a) {
+        constexpr int i = decltype(idx)::value;
+        constexpr Sum m = kList.s[2 * i];
+        if constexpr (2 * i + 2 == kSums) {
+            a.x = fmaf(m.row & 1 ? row[m.row / 2].y : row[m.row / 2].x, x[m.c] * x[m.d], a.x);
+            a.y += own;
+        } else {
+            float p = x[m.c];
+            if constexpr (m.d >= 0) p *= x[m.d];
+            a = __ffma2_rn(row[m.row / 2], make_float2(p, p), a);
+        }
     };
     (term(std::integral_constant<int, I>{}, acc[I]), ...);
 }
@@ -305,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
     __shared__ float s_c[7][kPix];             // the pixels' features
     __shared__ float s_s2[kNQ];                // squared natural-unit scale of each unknown
     __shared__ float s_d[kNA][kPix];           // equilibration scales
-    __shared__ float s_inv[7][kPix];           // 1 / diagonal of U_JJ
+    __shared__ float s_inv[kB][kPix];           // 1 / diagonal of U_JJ
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int pi = lane & 15, half = lane >> 4;
@@ -346,18 +377,22 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
     const float s_px = kExp2Scale / (p.h * (float)p.r);
     float* flushed = reinterpret_cast<float*>(sm) + warp * kPix + pi;           // of this warp and pixel, per sum
     float* table = reinterpret_cast<float*>(sm + (p.flush ? kFlushBytes : 0)) + lane;
-    float acc[kSums];
+    float2 acc[kSums / 2];
 #pragma unroll
-    for (int i = 0; i < kSums; ++i) acc[i] = 0.0f;
+    for (int i = 0; i < kSums / 2; ++i) acc[i] = make_float2(0.0f, 0.0f);
     int run = 0;             // pairs in the registers' partial sums
     bool any = false;        // partial sums have been flushed
-    auto flush = [&]() {     // add the halves, then to the flushed sums
+    auto both_halves = [&](float v) { return v + __shfl_xor_sync(0xffffffffu, v, 16); };
+    auto flush = [&]() {
 #pragma unroll
-        for (int i = 0; i < kSums; ++i) {
-            const float v = acc[i] + __shfl_xor_sync(0xffffffffu, acc[i], 16);
-            float* at = flushed + i * (kWarps * kPix);
-            if (half == 0) *at = any ? *at + v : v;
-            acc[i] = 0.0f;
+        for (int i = 0; i < kSums / 2; ++i) {
+            const float v[2] = {both_halves(acc[i].x), both_halves(acc[i].y)};
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float* at = flushed + (2 * i + h) * (kWarps * kPix);
+                if (half == 0) *at = any ? *at + v[h] : v[h];
+            }
+            acc[i] = make_float2(0.0f, 0.0f);
         }
         any = true;
         run = 0;
@@ -411,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
             for (int i = 0; i < m; ++i) {
                 const float x[8] = {ex[0], ex[32], ex[64], ex[96], ex[128], ex[160], ex[192], ex[224]};
                 add_sums(acc, e[kWz * 32], e[kWyz * 32], e[kZ * 32], ex[kWz * 32], x,
-                         std::make_integer_sequence<int, kSums>{});
+                         std::make_integer_sequence<int, kSums / 2>{});
                 e += kEntries * 32;
                 ex += kEntries * 32;
             }
@@ -421,9 +456,12 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
         __syncthreads();   // the table is free again
     }
 #pragma unroll
-    for (int i = 0; i < kSums; ++i) {
-        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
-        if (any) acc[i] += flushed[i * (kWarps * kPix)];
+    for (int i = 0; i < kSums / 2; ++i) {
+        acc[i] = make_float2(both_halves(acc[i].x), both_halves(acc[i].y));
+        if (any) {
+            acc[i].x += flushed[2 * i * (kWarps * kPix)];
+            acc[i].y += flushed[(2 * i + 1) * (kWarps * kPix)];
+        }
     }
     if (p.flush) __syncthreads();   // the matrix takes the place of the flushed sums
 
@@ -432,7 +470,7 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
     for (int i = 0; i < kSums; ++i) {
         const unsigned short* at = kPlaces.e[i][warp];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) mat[at[k] * kPix] = acc[i];
+        for (int k = 0; k < 3; ++k) mat[at[k] * kPix] = i & 1 ? acc[i / 2].y : acc[i / 2].x;
     }
     __syncthreads();
 
@@ -444,8 +482,7 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
             s_d[z][pi] = 1.0f;
             mat[elem(55, 55) * kPix] = 1.0f;
         } else {
-            const int J = z / 7, r = z - 7 * J;
-            float* at = mat + (tile_base(J, J) + diag_elem(r, r)) * kPix;
+            float* at = mat + elem(z, z) * kPix;
             const float a = z < 54 ? fmaf(lw, s_s2[z], *at) : *at;
             // lw is read by every warp: the intercept's entry stays as it is
             if (z < 54) *at = a;
@@ -454,94 +491,118 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
     }
     __syncthreads();
 
-    // ---- left-looking blocked Cholesky A = U^T U over 8 block columns of 7:
-    // in step J warp k forms tile (J, J + k) as A - sum_K U_KJ^T U_KL, warp 0
-    // factors the diagonal tile, the others solve theirs against it.  A lane
-    // holds 4 of its tile's columns: 0-3 in the first half, 3-6 in the second
-    // (an odd distance, so that the halves read different banks; column 3 is
-    // formed twice).
-    const int c0 = 3 * half;
-#pragma unroll 1
-    for (int J = 0; J < 8; ++J) {
-        const int L = J + warp;
-        float x[7][4];
-        if (L < 8) {
-            const bool diag = L == J;
-            {
-                float dc[4];
+    // ---- blocked Cholesky A = U^T U over 7 block columns of 8.  A warp forms one
+    // tile (I, L) as A - sum_K U_KI^T U_KL; a lane holds 4 of its columns, the
+    // even ones in the first half and the odd ones in the second (neighbouring
+    // elements lie in different banks).  Left-looking over block columns 0-3,
+    // then their part of the last six tiles at once (six warps, where the
+    // left-looking order would leave it to three, two and one), then
+    // left-looking over the rest.
+    constexpr int kSplit = 4;
+    float x[kB][4];
+    auto form = [&](int I, int L, int K0, int K1, bool scale) {
+        const float* A = mat + tile_base(I, L) * kPix;
+        float2 v[kB][2];
+        float dc[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) dc[k] = s_d[7 * L + c0 + k][pi];
-                const float* A = mat + tile_base(J, L) * kPix;
+        for (int k = 0; k < 4; ++k) dc[k] = scale ? -s_d[kB * L + 2 * k + half][pi] : -1.0f;
 #pragma unroll
-                for (int i = 0; i < 7; ++i) {
-                    const float dr = s_d[7 * J + i][pi];
+        for (int i = 0; i < kB; ++i) {
+            const float dr = scale ? s_d[kB * I + i][pi] : 1.0f;
+            float a[4];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int c = c0 + k;
-                        const int e = diag ? diag_elem(min(i, c), max(i, c)) : i * 7 + c;
-                        x[i][k] = A[e * kPix] * (dr * dc[k]);
-                    }
-                }
+            for (int k = 0; k < 4; ++k) {
+                const int c = 2 * k + half;
+                const int e = I == L ? diag_elem(min(i, c), max(i, c)) : i * kB + c;
+                a[k] = A[e * kPix] * (dr * dc[k]);
             }
+            v[i][0] = make_float2(a[0], a[1]);
+            v[i][1] = make_float2(a[2], a[3]);
+        }
 #pragma unroll 1
-            for (int K = 0; K < J; ++K) {
-                const float* UI = mat + tile_base(K, J) * kPix;
-                const float* UL = mat + (tile_base(K, L) + c0) * kPix;
+        for (int K = K0; K < K1; ++K) {
+            const float* UI = mat + tile_base(K, I) * kPix;
+            const float* UL = mat + (tile_base(K, L) + half) * kPix;
 #pragma unroll
-                for (int m = 0; m < 7; ++m) {
-                    float a[7], b[4];
+            for (int m = 0; m < kB; ++m) {
+                const float2 b0 = make_float2(UL[kB * m * kPix], UL[(kB * m + 2) * kPix]);
+                const float2 b1 = make_float2(UL[(kB * m + 4) * kPix], UL[(kB * m + 6) * kPix]);
 #pragma unroll
-                    for (int i = 0; i < 7; ++i) a[i] = UI[(7 * m + i) * kPix];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) b[k] = UL[(7 * m + k) * kPix];
-#pragma unroll
-                    for (int i = 0; i < 7; ++i)
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) x[i][k] = fmaf(-a[i], b[k], x[i][k]);
+                for (int i = 0; i < kB; ++i) {
+                    const float a = UI[(kB * m + i) * kPix];
+                    v[i][0] = __ffma2_rn(make_float2(a, a), b0, v[i][0]);
+                    v[i][1] = __ffma2_rn(make_float2(a, a), b1, v[i][1]);
                 }
-            }
-            if (diag) {
-                float* D = mat + tile_base(J, J) * kPix;
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 7; ++i)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (i <= c0 + k) D[diag_elem(i, c0 + k) * kPix] = x[i][k];
-                __syncwarp();
-                float g[28];
-#pragma unroll
-                for (int e = 0; e < 28; ++e) g[e] = D[e * kPix];
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 7; ++i) {
-                    const float piv = sqrtf(fmaxf(g[diag_elem(i, i)], 1e-30f));
-                    const float inv = 1.0f / piv;
-                    g[diag_elem(i, i)] = piv;
-#pragma unroll
-                    for (int k = i + 1; k < 7; ++k) g[diag_elem(i, k)] *= inv;
-#pragma unroll
-                    for (int m = i + 1; m < 7; ++m)
-#pragma unroll
-                        for (int k = m; k < 7; ++k)
-                            g[diag_elem(m, k)] = fmaf(-g[diag_elem(i, m)], g[diag_elem(i, k)], g[diag_elem(m, k)]);
-                    s_inv[i][pi] = inv;
-                }
-#pragma unroll
-                for (int e = 0; e < 28; ++e) D[e * kPix] = g[e];
-                // With the intercept last and y appended, U[54][55] = (U^-T b)_54 and
-                // theta_54 = U[54][55] / U[54][54] in the equilibrated basis.
-                if (J == 7 && half == 0 && px < p.W && py < p.H)
-                    p.alpha[(size_t)f * N + (size_t)py * p.W + px] =
-                        g[diag_elem(5, 6)] / g[diag_elem(5, 5)] * s_d[54][pi];
             }
         }
-        __syncthreads();
-        if (L < 8 && L > J) {
-            const float* D = mat + tile_base(J, J) * kPix;
-            float* X = mat + (tile_base(J, L) + c0) * kPix;
 #pragma unroll
-            for (int i = 0; i < 7; ++i) {
+        for (int i = 0; i < kB; ++i) {
+            x[i][0] = -v[i][0].x;
+            x[i][1] = -v[i][0].y;
+            x[i][2] = -v[i][1].x;
+            x[i][3] = -v[i][1].y;
+        }
+    };
+    auto put = [&](int I, int L) {
+        float* A = mat + tile_base(I, L) * kPix;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < kB; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int c = 2 * k + half;
+                if (I != L) A[(i * kB + c) * kPix] = x[i][k];
+                else if (i <= c) A[diag_elem(i, c) * kPix] = x[i][k];
+            }
+        __syncwarp();
+    };
+#pragma unroll 1
+    for (int J = 0; J < kNB; ++J) {
+        if (J == kSplit) {
+            if (warp < 6) {
+                const int I = warp < 3 ? 4 : warp < 5 ? 5 : 6, L = warp < 3 ? 4 + warp : warp < 5 ? 2 + warp : 6;
+                form(I, L, 0, kSplit, true);
+                put(I, L);
+            }
+            __syncthreads();
+        }
+        const int L = J + warp;
+        if (L < kNB) form(J, L, J < kSplit ? 0 : kSplit, J, J < kSplit);
+        if (warp == 0) {
+            // the diagonal tile, by every lane for its own pixel
+            put(J, J);
+            float* D = mat + tile_base(J, J) * kPix;
+            float g[kDiag];
+#pragma unroll
+            for (int e = 0; e < kDiag; ++e) g[e] = D[e * kPix];
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < kB; ++i) {
+                // 1 / sqrt of the pivot: one Newton step on the approximation
+                const float piv = fmaxf(g[diag_elem(i, i)], 1e-30f), r0 = rsqrtf(piv);
+                const float inv = fmaf(0.5f * r0, fmaf(-piv * r0, r0, 1.0f), r0);
+#pragma unroll
+                for (int k = i + 1; k < kB; ++k) g[diag_elem(i, k)] *= inv;
+#pragma unroll
+                for (int m = i + 1; m < kB; ++m)
+#pragma unroll
+                    for (int k = m; k < kB; ++k)
+                        g[diag_elem(m, k)] = fmaf(-g[diag_elem(i, m)], g[diag_elem(i, k)], g[diag_elem(m, k)]);
+                s_inv[i][pi] = inv;
+                // With the intercept last and y appended, U[54][55] = (U^-T b)_54 and
+                // theta_54 = U[54][55] / U[54][54] in the equilibrated basis.
+                if (i == kB - 2 && J == kNB - 1 && half == 0 && px < p.W && py < p.H)
+                    p.alpha[(size_t)f * N + (size_t)py * p.W + px] = g[diag_elem(i, i + 1)] * inv * s_d[54][pi];
+            }
+#pragma unroll
+            for (int e = 0; e < kDiag; ++e) D[e * kPix] = g[e];
+        }
+        if (J == kNB - 1) break;
+        __syncthreads();
+        if (L < kNB && L > J) {
+            const float* D = mat + tile_base(J, J) * kPix;
+#pragma unroll
+            for (int i = 0; i < kB; ++i) {
                 const float inv = s_inv[i][pi];
 #pragma unroll
                 for (int m = 0; m < i; ++m) {
@@ -552,11 +613,7 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) x[i][k] *= inv;
             }
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 7; ++i)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) X[(7 * i + k) * kPix] = x[i][k];
+            put(J, L);
         }
         __syncthreads();
     }
