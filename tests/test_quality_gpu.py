@@ -110,6 +110,19 @@ def test_quality_random_sets(shape, density):
     _compare(gen, ref)
 
 
+@pytest.mark.parametrize("shape,density", [((3, 32, 32), 0.03), ((2, 33, 33), 0.03), ((2, 31, 65), 0.01),
+                                           ((2, 4096, 3), 0.002), ((2, 4097, 3), 0.002)])
+def test_quality_column_pass_edges(shape, density):
+    """Whole and partial 32-row masks and 32-column blocks, the tallest image
+    with masks and one row past it; columns without any event."""
+    rng = np.random.default_rng(shape[1] + shape[2])
+    gen = rng.integers(-3, 4, size=shape) * (rng.random(shape) < density)
+    ref = rng.integers(-3, 4, size=shape) * (rng.random(shape) < density)
+    gen[:, :, 0] = 0
+    ref[:, :, -1] = 0
+    _compare(gen, ref)
+
+
 def test_quality_degenerate_sets():
     shape = (5, 8, 8)
     z = np.zeros(shape, np.int64)
