@@ -108,6 +108,40 @@ def test_gradients_match_oracle_finite_differences():
         assert g_rad[t, c, yy, xx].item() == pytest.approx(fd, rel=2e-3, abs=1e-7)
 
 
+@pytest.mark.parametrize("w,h,n,r,frames", [
+    (32, 8, 2, 3, 2),     # exactly one centre tile
+    (33, 9, 3, 2, 3),     # one pixel past it
+    (7, 5, 3, 3, 2),      # an image smaller than the window
+    (70, 20, 2, 4, 2),    # three tiles across and down
+    (36, 20, 3, 9, 3),    # tile sums larger than the workspace: the gather over the centres
+])
+def test_radiance_gradient_paths(w, h, n, r, frames):
+    from paper_2303_02608_gb300 import wlr
+    rad, feat, clean = _crop(RECTS, 20, 30, w, h, n)
+    rd = rad.cuda().requires_grad_(True)
+    bd = torch.tensor(B, dtype=torch.float32, device="cuda", requires_grad=True)
+    alpha = wlr(rd, feat.cuda(), bd, radius=r, frames=frames, log_eps=EPS, ridge=RIDGE)
+    ((alpha - log_luminance(clean.cuda(), EPS)) ** 2).mean().backward()
+    r64, b64 = rad.double().requires_grad_(True), torch.tensor(B, dtype=torch.float64, requires_grad=True)
+    mse_loss(wlr_alpha(r64, feat.double(), b64, r, frames, eps=EPS, ridge=RIDGE), clean.double(), EPS).backward()
+    gb, gr = b64.grad.numpy(), r64.grad.numpy()
+    np.testing.assert_allclose(bd.grad.cpu().numpy(), gb, rtol=2e-3, atol=2e-3 * np.abs(gb).max())
+    np.testing.assert_allclose(rd.grad.cpu().numpy(), gr, rtol=1e-4, atol=1e-5 * np.abs(gr).max())
+
+
+def test_masked_centres_add_nothing():
+    """Centres whose alpha the loss leaves out contribute nothing, even where
+    their inputs are not numbers."""
+    from paper_2303_02608_gb300 import wlr
+    rad, feat, _ = _crop(RECTS, 20, 30, 40, 16, 1)
+    rad[0, :, 0, 0] = float("nan")
+    rd = rad.cuda().requires_grad_(True)
+    bd = torch.tensor(B, dtype=torch.float32, device="cuda", requires_grad=True)
+    wlr(rd, feat.cuda(), bd, radius=R, frames=1)[0, :, 20:].sum().backward()
+    assert torch.isfinite(bd.grad).all()
+    assert torch.isfinite(rd.grad[:, :, :, 17:]).all() and not rd.grad[0, :, :, 4:10].any()
+
+
 def test_backward_is_deterministic():
     rad, feat, clean = _crop(RECTS, 0, 0, 64, 48, 4)
     a = _gpu(rad, feat, clean, B)
