@@ -813,13 +813,14 @@ esim_ad_status esim_ad_batch_denoised(esim_ad_batch* b, int32_t seq, float* alph
                                       int dst_is_device)
 {
     if (!b || seq < 0 || seq >= b->n) return ESIM_AD_EINVAL;
-    const cudaMemcpyKind k = dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    const size_t N = b->N[seq];
-    if ((alpha && cudaMemcpyAsync(alpha, b->alpha[seq], N * sizeof(float), k, b->stream) != cudaSuccess) ||
-        (flags && cudaMemcpyAsync(flags, b->flag[seq], N, k, b->stream) != cudaSuccess) ||
-        cudaStreamSynchronize(b->stream) != cudaSuccess)
-        return ESIM_AD_ECUDA;
-    return ESIM_AD_OK;
+    int prev = -1;
+    cudaGetDevice(&prev);
+    if (prev != b->device) cudaSetDevice(b->device);
+    const bool ok = copy_maps(b->alpha[seq], alpha, b->flag[seq], flags, b->N[seq], dst_is_device != 0, b->device,
+                              b->stream) == cudaSuccess &&
+                    cudaStreamSynchronize(b->stream) == cudaSuccess;
+    if (prev >= 0 && prev != b->device) cudaSetDevice(prev);
+    return ok ? ESIM_AD_OK : ESIM_AD_ECUDA;
 }
 
 esim_ad_status esim_ad_batch_get_state(esim_ad_batch* b, int32_t seq, float* l_last, float* beta, float* xc)

@@ -68,7 +68,7 @@ struct esim_ad_ctx {
     // that frame's writer only, not for the frames pushed after it
     cudaStream_t drain_stream = nullptr;
     uint64_t drained = 0;                 // event positions drained so far
-    unsigned long long* hmark = nullptr;  // pinned: a frame's end mark and the status word
+    HostMarks* marks = nullptr;           // pinned, written by the event writers
     int device = 0;
     int W = 0, H = 0;
     size_t N = 0;
@@ -173,7 +173,7 @@ void release(esim_ad_ctx* c)
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
     if (c->writer_stream) cudaStreamDestroy(c->writer_stream);
     if (c->drain_stream) cudaStreamDestroy(c->drain_stream);
-    if (c->hmark) cudaFreeHost(c->hmark);
+    if (c->marks) cudaFreeHost(c->marks);
     if (c->ev_solved) cudaEventDestroy(c->ev_solved);
     for (cudaEvent_t e : c->ev_wr)
         if (e) cudaEventDestroy(e);
@@ -282,16 +282,38 @@ esim_ad_status encode_ring_map(esim_ad_ctx* c)
                : ESIM_AD_ECUDA;
 }
 
-esim_ad_status sync_and_check(esim_ad_ctx* c, Ctrl* host_ctrl)
+void note_status(esim_ad_ctx* c, uint32_t status)
 {
-    Ctrl tmp;
-    Ctrl* h = host_ctrl ? host_ctrl : &tmp;
+    if (status & kStatusTimeout) c->sticky = ESIM_AD_ETIMEOUT;
+    else if (status & kStatusOverflow) c->sticky = ESIM_AD_EOVERFLOW;
+}
+
+uint32_t marked_status(const esim_ad_ctx* c)
+{
+    const volatile HostMarks* m = c->marks;
+    return m->status | (m->overflow ? kStatusOverflow : 0u);
+}
+
+esim_ad_status sync_and_check(esim_ad_ctx* c, Ctrl* h)
+{
     if (join_writer(c) != cudaSuccess ||
         cudaMemcpyAsync(h, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
         return ESIM_AD_ECUDA;
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return ESIM_AD_ECUDA;
-    if (h->status & kStatusTimeout) c->sticky = ESIM_AD_ETIMEOUT;
-    else if (h->status & kStatusOverflow) c->sticky = ESIM_AD_EOVERFLOW;
+    note_status(c, h->status);
+    return ESIM_AD_OK;
+}
+
+// The same where only the status is wanted: a context whose latest frame has a
+// writer (frame 0 has none) finds it in the writer's marks.
+esim_ad_status sync_and_check(esim_ad_ctx* c)
+{
+    if (c->t < 2) {
+        Ctrl h;
+        return sync_and_check(c, &h);
+    }
+    if (sync_stream(c) != cudaSuccess) return ESIM_AD_ECUDA;
+    note_status(c, marked_status(c));
     return ESIM_AD_OK;
 }
 
@@ -388,7 +410,7 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
             return cudaStreamCreateWithPriority(&c->writer_stream, cudaStreamNonBlocking, hi) == cudaSuccess;
         }() == false ||
         cudaStreamCreateWithFlags(&c->drain_stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaHostAlloc((void**)&c->hmark, 2 * sizeof(unsigned long long), cudaHostAllocDefault) != cudaSuccess ||
+        cudaHostAlloc((void**)&c->marks, sizeof(HostMarks), cudaHostAllocMapped) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_solved, cudaEventDisableTiming) != cudaSuccess ||
         [&] {
             for (cudaEvent_t& e : c->ev_wr)
@@ -400,6 +422,7 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
         delete c;
         return ESIM_AD_ECUDA;
     }
+    memset(c->marks, 0, sizeof(HostMarks));
     {
         const int sp = wlr_sparse_smem(cfg->radius, c->mixed);
         c->smem_adaptive = c->smem_bytes > sp ? c->smem_bytes : sp;
@@ -682,6 +705,7 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
         ep.chunk_off = c->chunk_off;
         ep.events = c->events;
         ep.capacity = c->cfg.event_capacity;
+        ep.marks = c->marks;
         ep.ctrl = c->ctrl;
         // on the writer stream, so that the next frame's ingest and pass 1 run
         // beside it; while profiling, on the context's stream, so that every
@@ -760,26 +784,22 @@ esim_ad_status esim_ad_events_frame(esim_ad_ctx* c, uint64_t frame, esim_ad_even
     if (c->sticky != ESIM_AD_OK) return ESIM_AD_ESTATE;
     if (frame >= c->t || c->t - 1 - frame >= (uint64_t)kFrameEnds) return ESIM_AD_EINVAL;
     DeviceGuard guard(c->device);
-    // wait for that frame's writer only, on the drain stream; its end mark and
-    // the status word land in pinned memory
-    struct {
-        unsigned long long end;
-        uint32_t status;
-    } h = {0, 0};
-    const cudaStream_t s = c->drain_stream;
-    c->hmark[1] = 0;
-    if (cudaStreamWaitEvent(s, c->ev_wr[frame % kFrameEnds], 0) != cudaSuccess ||
-        cudaMemcpyAsync(&c->hmark[0], &c->ctrl->frame_end[frame % kFrameEnds], sizeof(unsigned long long),
-                        cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(&c->hmark[1], &c->ctrl->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
+    // wait for that frame's writer only; its end mark and the status are in host
+    // memory by then
+    unsigned long long end = c->drained;   // frame 0 writes no events (and no marks)
+    uint32_t status = 0;
+    if (frame > 0) {
+        if (cudaEventSynchronize(c->ev_wr[frame % kFrameEnds]) != cudaSuccess) return ESIM_AD_ECUDA;
+        end = static_cast<volatile HostMarks*>(c->marks)->frame_end[frame % kFrameEnds];
+        status = marked_status(c);
+    } else if (cudaStreamWaitEvent(c->drain_stream, c->ev_wr[0], 0) != cudaSuccess ||
+               cudaMemcpyAsync(&status, &c->ctrl->status, sizeof(status), cudaMemcpyDeviceToHost, c->drain_stream) !=
+                   cudaSuccess ||
+               cudaStreamSynchronize(c->drain_stream) != cudaSuccess) {
         return ESIM_AD_ECUDA;
-    h.end = c->hmark[0];
-    h.status = (uint32_t)c->hmark[1];
-    if (frame == 0) h.end = c->drained;   // frame 0 writes no events (and no end mark)
-    if (h.status & kStatusTimeout) c->sticky = ESIM_AD_ETIMEOUT;
-    else if (h.status & kStatusOverflow) c->sticky = ESIM_AD_EOVERFLOW;
-    const unsigned long long n = h.end > c->drained ? h.end - c->drained : 0ull;
+    }
+    note_status(c, status);
+    const unsigned long long n = end > c->drained ? end - c->drained : 0ull;
     if (c->sticky == ESIM_AD_EOVERFLOW) {
         *n_out = n;
         return ESIM_AD_EOVERFLOW;
@@ -787,7 +807,7 @@ esim_ad_status esim_ad_events_frame(esim_ad_ctx* c, uint64_t frame, esim_ad_even
     if (c->sticky != ESIM_AD_OK) return c->sticky;
     *n_out = n;
     if (cap < n) return ESIM_AD_ENOSPACE;
-    return n > 0 ? copy_ring(c, dst, c->drained, n, dst_is_device, s) : ESIM_AD_OK;
+    return n > 0 ? copy_ring(c, dst, c->drained, n, dst_is_device, c->drain_stream) : ESIM_AD_OK;
 }
 
 esim_ad_status esim_ad_denoised(esim_ad_ctx* c, float* alpha, uint8_t* flags, int dst_is_device)
@@ -795,11 +815,9 @@ esim_ad_status esim_ad_denoised(esim_ad_ctx* c, float* alpha, uint8_t* flags, in
     if (!c) return ESIM_AD_EINVAL;
     if (c->sticky != ESIM_AD_OK) return ESIM_AD_ESTATE;
     DeviceGuard guard(c->device);
-    const cudaMemcpyKind k = dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (alpha && cudaMemcpyAsync(alpha, c->alpha, c->N * sizeof(float), k, c->stream) != cudaSuccess)
+    if (copy_maps(c->alpha, alpha, c->flag, flags, c->N, dst_is_device != 0, c->device, c->stream) != cudaSuccess)
         return ESIM_AD_ECUDA;
-    if (flags && cudaMemcpyAsync(flags, c->flag, c->N, k, c->stream) != cudaSuccess) return ESIM_AD_ECUDA;
-    if (sync_and_check(c, nullptr) != ESIM_AD_OK) return ESIM_AD_ECUDA;
+    if (sync_and_check(c) != ESIM_AD_OK) return ESIM_AD_ECUDA;
     return c->sticky == ESIM_AD_OK ? ESIM_AD_OK : c->sticky;
 }
 
@@ -812,7 +830,7 @@ esim_ad_status esim_ad_get_state(esim_ad_ctx* c, float* l_last, float* beta, flo
     float4* h = (float4*)malloc(4 * N * sizeof(float4));
     if (!h) return ESIM_AD_ENOMEM;
     if (cudaMemcpyAsync(h, c->state, 4 * N * sizeof(float4), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
-        sync_and_check(c, nullptr) != ESIM_AD_OK) {
+        sync_and_check(c) != ESIM_AD_OK) {
         free(h);
         return ESIM_AD_ECUDA;
     }
@@ -880,6 +898,7 @@ esim_ad_status esim_ad_reset(esim_ad_ctx* c)
     if (cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream) != cudaSuccess ||
         sync_stream(c) != cudaSuccess)
         return ESIM_AD_ECUDA;
+    memset(c->marks, 0, sizeof(HostMarks));
     c->t = 0;
     c->drained = 0;
     c->staged_ingests = 0;

@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(kThreads) event_write_kernel(EventParams p)
     }
     const unsigned long long drained = p.drained;
     const unsigned long long before = p.ctrl->ev_base + block_prefix_count(p.chunk_cnt, blockIdx.x, s_red);
-    const bool range_ok = (p.ctrl->status & kStatusCountRange) == 0u;
+    const uint32_t status = p.ctrl->status;
+    const bool range_ok = (status & kStatusCountRange) == 0u;
     if (last && threadIdx.x == 0) {
         if (!range_ok) {
             p.ctrl->ev_total = ~0ull;   // the map was out of range: nothing is written
@@ -98,6 +99,10 @@ __global__ void __launch_bounds__(kThreads) event_write_kernel(EventParams p)
             p.ctrl->ev_total = before + cnt;
             p.ctrl->ev_cum += before + cnt - p.ctrl->ev_base;
             p.ctrl->frame_end[p.frame % kFrameEnds] = before + cnt;
+            if (p.marks) {
+                p.marks->frame_end[p.frame % kFrameEnds] = before + cnt;
+                p.marks->status = status;
+            }
         }
     }
     if (cnt == 0u || !range_ok) return;
@@ -139,7 +144,10 @@ __global__ void __launch_bounds__(kThreads) event_write_kernel(EventParams p)
             if (++idx == p.capacity) idx = 0;
         }
     }
-    if (overflow) atomicOr(&p.ctrl->status, kStatusOverflow);
+    if (overflow) {
+        atomicOr(&p.ctrl->status, kStatusOverflow);
+        if (p.marks) p.marks->overflow = 1u;
+    }
 }
 
 }  // namespace

@@ -179,6 +179,14 @@ struct WlrParams {
     Ctrl* ctrl;
 };
 
+// What a drain needs to know of a frame, in host memory that the writer fills
+// itself: read after the writer's event, it costs no copy.
+struct HostMarks {
+    unsigned long long frame_end[kFrameEnds];   // as Ctrl::frame_end
+    uint32_t status;                            // Ctrl::status as the latest writer began
+    uint32_t overflow;                          // some writer dropped records
+};
+
 struct EventParams {
     const int32_t* nev;
     const uint32_t* ev_mask = nullptr;   // bit per pixel with events (nullptr: read every count)
@@ -191,6 +199,7 @@ struct EventParams {
     unsigned long long* chunk_off;
     esim_ad_event* events;
     unsigned long long capacity;
+    HostMarks* marks = nullptr;          // simulator's writer
     Ctrl* ctrl;
 };
 
@@ -221,6 +230,9 @@ cudaError_t launch_wlr(const CUtensorMap& tmap, const WlrParams& p, bool mixed, 
 cudaError_t launch_wlr_solve(const WlrParams& p, bool mixed, int grid, cudaStream_t s);
 int wlr_solve_grid(int num_sms);
 cudaError_t launch_events(const EventParams& p, cudaStream_t s);
+// Copy a frame's n-pixel maps (either may be null) to the caller's buffers.
+cudaError_t copy_maps(const float* alpha, float* alpha_out, const uint8_t* flag, uint8_t* flag_out, size_t n,
+                      bool to_device, int device, cudaStream_t s);
 cudaError_t launch_event_write(const EventParams& p, cudaStream_t s);
 
 }  // namespace esim
