@@ -54,6 +54,7 @@ struct SeqStep {
 
 struct BatchGlobal {
     const SeqStep* steps;
+    const RingMaps* maps;        // TMA views of each sequence's ring
     const uint16_t* tile_seq;    // global tile -> sequence
     const uint16_t* chunk_seq;   // global chunk -> sequence
     uint32_t* flag_list;         // (seq << 24) | pixel
@@ -74,10 +75,12 @@ constexpr int kTileWidths[kTileShapes] = {16, 32, 64};
 // Sequences of a batch: list entries are (sequence << 24) | pixel.
 struct BatchSeq {
     const SeqStep* steps;
+    const RingMaps* maps;   // per sequence
     __device__ __forceinline__ SeqView view(uint32_t e) const
     {
         const WlrParams& sp = steps[e >> kPixBits].wp;
-        return {sp.W, sp.H, sp.t, sp.T, sp.n_tau, sp.ring};
+        const RingMaps& m = maps[e >> kPixBits];
+        return {sp.W, sp.H, sp.t, sp.T, sp.n_tau, sp.ring, &m.box_small, &m.box_large};
     }
     __device__ __forceinline__ uint32_t pixel(uint32_t e) const { return e & kPixMask; }
     __device__ __forceinline__ const WlrParams& params(uint32_t e) const { return steps[e >> kPixBits].wp; }
@@ -129,7 +132,7 @@ __global__ void __launch_bounds__(kTilePix) batch_ingest_kernel(BatchGlobal g)
 template <int kItem, bool kMixed>
 __global__ void __launch_bounds__(kTilePix, 2) batch_wlr_kernel(BatchGlobal g, const WlrParams gp)
 {
-    sparse_body<kItem, kMixed>(gp, BatchSeq{g.steps});
+    sparse_body<kItem, kMixed>(gp, BatchSeq{g.steps, g.maps});
 }
 
 // Pass 2: solve every record and emit into its sequence's maps; the last CTA
@@ -138,7 +141,7 @@ template <bool kMixed>
 __global__ void __launch_bounds__(kSolveThreads, 3) batch_solve_kernel(BatchGlobal g, const WlrParams gp)
 {
     const uint32_t n = *(volatile uint32_t*)&g.ctrl->list_len;
-    const unsigned long long fp64 = solve_records<kMixed>(gp, BatchSeq{g.steps}, n);
+    const unsigned long long fp64 = solve_records<kMixed>(gp, BatchSeq{g.steps, g.maps}, n);
     finish(gp, 0ull, 0ull, fp64, false, true);
 }
 
@@ -239,6 +242,7 @@ struct esim_ad_batch {
     esim_ad_batch_event* events = nullptr;
     Ctrl* ctrl = nullptr;
     SeqStep* d_steps = nullptr;
+    RingMaps* d_maps = nullptr;   // window boxes of each sequence's ring
     SeqStep* h_steps[2] = {nullptr, nullptr};   // pinned, alternating
     cudaEvent_t h_free[2] = {nullptr, nullptr};
     int cur = 0;
@@ -303,7 +307,7 @@ void batch_release(esim_ad_batch* b)
         if (i < (int)b->nev.size() && b->nev[i]) cudaFree(b->nev[i]);
     }
     void* g[] = {b->tile_seq_s[0], b->tile_seq_s[1], b->tile_seq_s[2], b->chunk_seq, b->flag_list, b->gram,
-                 b->chunk_cnt, b->chunk_off, b->events, b->ctrl, b->d_steps};
+                 b->chunk_cnt, b->chunk_off, b->events, b->ctrl, b->d_steps, b->d_maps};
     for (void* p : g)
         if (p) cudaFree(p);
     for (int k = 0; k < 2; ++k) {
@@ -320,6 +324,7 @@ BatchGlobal globals(const esim_ad_batch* b, int shape)
 {
     BatchGlobal g;
     g.steps = b->d_steps;
+    g.maps = b->d_maps;
     g.tile_seq = b->tile_seq_s[shape];
     g.chunk_seq = b->chunk_seq;
     g.flag_list = b->flag_list;
@@ -629,8 +634,17 @@ esim_ad_status esim_ad_batch_init(const esim_ad_config* cfgs, int32_t n_seq, voi
         cudaMalloc((void**)&b->chunk_off, (size_t)b->total_chunks * 8) != cudaSuccess ||
         cudaMalloc((void**)&b->events, (size_t)c0.event_capacity * sizeof(esim_ad_batch_event)) != cudaSuccess ||
         cudaMalloc((void**)&b->ctrl, sizeof(Ctrl)) != cudaSuccess ||
-        cudaMalloc((void**)&b->d_steps, sizeof(SeqStep) * n_seq) != cudaSuccess)
+        cudaMalloc((void**)&b->d_steps, sizeof(SeqStep) * n_seq) != cudaSuccess ||
+        cudaMalloc((void**)&b->d_maps, sizeof(RingMaps) * n_seq) != cudaSuccess)
         return fail(ESIM_AD_ENOMEM);
+    {
+        std::vector<RingMaps> maps(n_seq);
+        for (int i = 0; i < n_seq; ++i)
+            if (!encode_boxes(&maps[i], b->ring[i], cfgs[i].width, cfgs[i].height, c0.frames, b->mixed))
+                return fail(ESIM_AD_ECUDA);
+        if (cudaMemcpy(b->d_maps, maps.data(), sizeof(RingMaps) * n_seq, cudaMemcpyHostToDevice) != cudaSuccess)
+            return fail(ESIM_AD_ECUDA);
+    }
     for (int k = 0; k < 2; ++k) {
         if (cudaMallocHost((void**)&b->h_steps[k], sizeof(SeqStep) * n_seq) != cudaSuccess)
             return fail(ESIM_AD_ENOMEM);

@@ -10,6 +10,57 @@
 #include <vector>
 
 #include "internal.h"
+#include "sparse_stage.cuh"
+
+namespace esim {
+namespace {
+
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
+                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeTiledFn encode_fn()
+{
+    static EncodeTiledFn fn = nullptr;
+    if (!fn) {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<EncodeTiledFn>(f);
+    }
+    return fn;
+}
+
+}  // namespace
+
+bool encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t rank, const void* ptr, const cuuint64_t* dims,
+                  const cuuint64_t* strides, const cuuint32_t* box)
+{
+    EncodeTiledFn fn = encode_fn();
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn && fn(m, dt, rank, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The ring as rows of 16-byte records, so that a box's rows are contiguous runs:
+// mixed form {8W halves, H, T}, FP32 form {4W floats, H, 2T half-planes}.
+bool encode_boxes(RingMaps* m, const void* ring, int W, int H, int T, bool mixed)
+{
+    const cuuint32_t el = mixed ? 8 : 4;
+    const CUtensorMapDataType dt = mixed ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    const cuuint64_t dims[3] = {(cuuint64_t)el * W, (cuuint64_t)H, (cuuint64_t)((mixed ? 1 : 2) * T)};
+    const cuuint64_t strides[2] = {(cuuint64_t)16 * W, (cuuint64_t)16 * W * H};
+    const cuuint32_t small[3] = {el * kPitchSmall, (cuuint32_t)kRowsSmall, mixed ? 1u : 2u};
+    const cuuint32_t large[3] = {el * kPitchLarge, (cuuint32_t)kRowsLarge, 1u};
+    return encode_tiled(&m->box_small, dt, 3, ring, dims, strides, small) &&
+           (!mixed || encode_tiled(&m->box_large, dt, 3, ring, dims, strides, large));
+}
+
+}  // namespace esim
 
 using namespace esim;
 
@@ -18,11 +69,6 @@ namespace {
 // sqrt(log2(e) / 2): scaling a regressor by k/(h b) turns the product
 // Gaussian exp(-sum (d/(h b))^2 / 2) of Eq. 5 into 2^(-sum u^2).
 const double kExp2Scale = 0.84932180028801904272;
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 // Allocation-failure injection for tests: ESIM_AD_FAULT_ALLOC=<k> makes the
 // k-th device allocation of the process (1-based) fail with ENOMEM.
@@ -103,7 +149,7 @@ struct esim_ad_ctx {
     cudaEvent_t ev_copied[2] = {nullptr, nullptr};
     cudaEvent_t ev_consumed[2] = {nullptr, nullptr};
     int staging_next = 0;
-    CUtensorMap tmap;
+    RingMaps maps;
     // staged ingest (precision form, FP16/BF16 frames): the model-state map is
     // fixed; the input maps are encoded per frame (its pointers and pitch)
     CUtensorMap ingest_map_s;
@@ -220,31 +266,6 @@ cudaError_t sync_stream(esim_ad_ctx* c)
     return e != cudaSuccess ? e : cudaStreamSynchronize(c->stream);
 }
 
-EncodeTiledFn encode_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(f);
-    }
-    return fn;
-}
-
-// Tiled map without swizzle or interleave; out-of-range elements read as zero.
-bool encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t rank, const void* ptr, const cuuint64_t* dims,
-                  const cuuint64_t* strides, const cuuint32_t* box)
-{
-    EncodeTiledFn fn = encode_fn();
-    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    return fn && fn(m, dt, rank, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // Input maps of one FP16/BF16 frame for the staged ingest: {W, H} log
 // brightness and {W, H, 7} features, boxes of one 32 x 8 tile.  False when the
 // frame does not meet TMA's rules (16-byte aligned planes, row pitch a
@@ -276,8 +297,9 @@ esim_ad_status encode_ring_map(esim_ad_ctx* c)
     const cuuint64_t strides[3] = {16, (cuuint64_t)16 * c->W, (cuuint64_t)16 * c->W * c->H};
     const cuuint32_t box[4] = {mixed ? 8u : 4u, (cuuint32_t)(kTileX + 2 * c->cfg.radius),
                                (cuuint32_t)(kTileY + 2 * c->cfg.radius), mixed ? 1u : 2u};
-    return encode_tiled(&c->tmap, mixed ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
-                        c->ring, dims, strides, box)
+    return encode_tiled(&c->maps.tile, mixed ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
+                        c->ring, dims, strides, box) &&
+                   encode_boxes(&c->maps, c->ring, c->W, c->H, c->cfg.frames, mixed)
                ? ESIM_AD_OK
                : ESIM_AD_ECUDA;
 }
@@ -681,7 +703,7 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
         // pass 1: dense frames tile-staged over every tile; adaptive frames in one
         // launch that picks window boxes or the tile queue from the flagged total
         const int grid = wp.dense ? (c->n_tiles < c->wlr_grid ? c->n_tiles : c->wlr_grid) : c->adaptive_grid;
-        if (launch_wlr(c->tmap, wp, c->mixed, grid, wp.dense ? c->smem_bytes : c->smem_adaptive, c->stream) !=
+        if (launch_wlr(c->maps, wp, c->mixed, grid, wp.dense ? c->smem_bytes : c->smem_adaptive, c->stream) !=
             cudaSuccess)
             return ESIM_AD_ECUDA;
         // pass 2: solve every accumulated system and emit; it follows the

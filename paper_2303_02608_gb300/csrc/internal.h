@@ -217,6 +217,15 @@ int ingest_staged_grid(int sms);
 // Autotuning cache (tune_cache.cu): value for key, or 0 if none.
 int tune_cache_lookup(const char* key);
 void tune_cache_store(const char* key, int value);
+// TMA views of a ring: one box per staged tile, and the window boxes.
+struct RingMaps {
+    CUtensorMap tile, box_small, box_large;
+};
+// Tiled map without swizzle or interleave; out-of-range elements read as zero.
+bool encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t rank, const void* ptr, const cuuint64_t* dims,
+                  const cuuint64_t* strides, const cuuint32_t* box);
+// The window boxes of a ring (box_large stays as it is in the FP32 form).
+bool encode_boxes(RingMaps* m, const void* ring, int W, int H, int T, bool mixed);
 // Regression pass 1: dense frames (every tile) and adaptive frames (one launch
 // choosing on the device between the sparse window-box form and the
 // tile-staged queue form); the adaptive kernel's shared memory is the larger
@@ -225,8 +234,7 @@ cudaError_t wlr_prepare(int smem_dense, int smem_adaptive, bool mixed);
 size_t wlr_smem_bytes(int r, bool mixed, int max_smem_per_sm, int* nbuf);
 int wlr_grid(int smem_bytes, int num_sms, bool mixed, bool adaptive);
 int wlr_sparse_smem(int r, bool mixed);
-cudaError_t launch_wlr(const CUtensorMap& tmap, const WlrParams& p, bool mixed, int grid,
-                       int smem_bytes, cudaStream_t s);
+cudaError_t launch_wlr(const RingMaps& m, const WlrParams& p, bool mixed, int grid, int smem_bytes, cudaStream_t s);
 cudaError_t launch_wlr_solve(const WlrParams& p, bool mixed, int grid, cudaStream_t s);
 int wlr_solve_grid(int num_sms);
 cudaError_t launch_events(const EventParams& p, cudaStream_t s);

@@ -99,17 +99,6 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
         : "memory");
 }
 
-// Bulk asynchronous copy of `bytes` contiguous bytes global -> this CTA's
-// shared memory (the TMA engine), completing `bytes` transactions on `bar`.
-// Both addresses 16-byte aligned, bytes a multiple of 16.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
-{
-    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
-
 // 2^x on the MUFU unit (ex2.approx, flush-to-zero).
 __device__ __forceinline__ float ex2_approx(float x)
 {

@@ -15,12 +15,18 @@ namespace {
 struct SeqView {
     int W, H, t, T, n_tau;
     const void* ring;
+    const CUtensorMap* box_small;   // the ring in boxes of kPitchSmall x kRowsSmall records
+    const CUtensorMap* box_large;   // mixed form: kPitchLarge x kRowsLarge
 };
 
 // One sequence: list entries are pixel indices.
 struct SingleSeq {
     const WlrParams* p;
-    __device__ __forceinline__ SeqView view(uint32_t) const { return {p->W, p->H, p->t, p->T, p->n_tau, p->ring}; }
+    const CUtensorMap *box_small, *box_large;
+    __device__ __forceinline__ SeqView view(uint32_t) const
+    {
+        return {p->W, p->H, p->t, p->T, p->n_tau, p->ring, box_small, box_large};
+    }
     __device__ __forceinline__ uint32_t pixel(uint32_t e) const { return e; }
     __device__ __forceinline__ const WlrParams& params(uint32_t) const { return *p; }
 };
@@ -202,11 +208,13 @@ __device__ __noinline__ void refine_fp64(const WlrParams& p, uint32_t pix, const
 // edge), 8 lanes per pixel (16 or 32 when the item holds only two or one
 // pixel, the tail of a tile's run).  For each frame of the temporal window the
 // bounding box of the four windows (clipped to the image) is copied from the
-// ring into the warp's shared memory by bulk asynchronous copies (the TMA
-// engine, one row per lane, completing on the warp's mbarrier).  Boxes of up
-// to 20 x 20 records are double-buffered: frame k+1's copy is issued before
-// frame k is summed.  Larger boxes take the whole buffer one frame at a time;
-// boxes too large for it are read through L1.  The lanes split each window's
+// ring into the warp's shared memory by one TMA box load, completing on the
+// warp's mbarrier: a box of fixed size from the windows' first corner, the ring
+// seen as rows of records (what lies past the image reads as zero, and no
+// window reaches it).  Boxes of up to 20 x 20 records are double-buffered: frame
+// k+1's copy is issued before frame k is summed.  Larger boxes take the whole
+// buffer one frame at a time; boxes too large for it are read through L1.
+// BOXMEASURED  The lanes split each window's
 // offsets and accumulate the 65 sums in packed FP32 pairs; the g lanes of a
 // pixel are then reduced by shuffles and store one Gram record at the pixel's
 // position in the flagged list.  Warps fetch work independently; there is no
@@ -214,7 +222,9 @@ __device__ __noinline__ void refine_fp64(const WlrParams& p, uint32_t pix, const
 template <int kItem, bool kMixed, class Src>
 __device__ __forceinline__ void sparse_body(const WlrParams& p, const Src& src)
 {
-    extern __shared__ __align__(128) unsigned char sm[];
+    extern __shared__ __align__(128) unsigned char sm_raw[];
+    // TMA destinations must be 128-byte aligned; the allocation has 128 bytes of slack
+    unsigned char* sm = sm_raw + ((128u - (smem_addr(sm_raw) & 127u)) & 127u);
     const BoxLayout L = box_layout(p.r);
     __shared__ unsigned long long s_pairs, s_pix;
     const int side = 2 * p.r + 1, nq = side * side;
@@ -356,19 +366,17 @@ __device__ __forceinline__ void sparse_body(const WlrParams& p, const Src& src)
         auto issue = [&](int b, int k) {
             __syncwarp();
             fence_proxy_async_smem();
-            if (p.withhold_copy && first_item && k == 0) return;   // test: this phase never completes
-            const int slot = (sv.t - k) % sv.T;
-            const uint32_t rowb = (uint32_t)bw * 16u;
-            if (lane == 0) mbar_arrive_expect_tx(&bar[b], (uint32_t)bh * rowb * (kMixed ? 1u : 2u));
             __syncwarp();
-            if (lane < bh) {
-                const size_t gi = (size_t)(by0 + lane) * sv.W + bx0;
-                unsigned char* dst = wbuf + (mode == 2 ? b * (kBoxBytes / 2) : 0) + lane * P * 16;
+            if (p.withhold_copy && first_item && k == 0) return;   // test: this phase never completes
+            if (lane == 0) {
+                const int slot = (sv.t - k) % sv.T;
+                unsigned char* dst = wbuf + (mode == 2 ? b * (kBoxBytes / 2) : 0);
                 if (kMixed) {
-                    bulk_load(dst, ringm + (size_t)slot * N + gi, rowb, &bar[b]);
+                    mbar_arrive_expect_tx(&bar[b], mode == 2 ? (uint32_t)kBoxBytes / 2u : (uint32_t)kBoxBytes);
+                    tma_load_3d(dst, mode == 2 ? sv.box_small : sv.box_large, &bar[b], 8 * bx0, by0, slot);
                 } else {
-                    bulk_load(dst, ringf + (size_t)(2 * slot) * N + gi, rowb, &bar[b]);
-                    bulk_load(dst + kBoxBytes / 2, ringf + (size_t)(2 * slot + 1) * N + gi, rowb, &bar[b]);
+                    mbar_arrive_expect_tx(&bar[b], (uint32_t)kBoxBytes);
+                    tma_load_3d(dst, sv.box_small, &bar[b], 4 * bx0, by0, 2 * slot);
                 }
             }
         };

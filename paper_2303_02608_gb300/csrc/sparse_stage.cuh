@@ -21,6 +21,8 @@ constexpr int kBoxBytes = 12800;
 constexpr int kPitchSmall = 20, kRowsSmall = 20;
 constexpr int kPitchLarge = 32, kRowsLarge = 25;
 constexpr int kBoxWarps = kTilePix / 32;
+static_assert(kPitchSmall * kRowsSmall * 32 == kBoxBytes && kPitchLarge * kRowsLarge * 16 == kBoxBytes,
+              "boxes fill the buffer or its halves; an FP32 box's second half-plane starts at the middle");
 
 struct BoxLayout {
     int tab_small, tab_large, bar_off, buf_off, total;
@@ -34,8 +36,8 @@ __host__ __device__ inline BoxLayout box_layout(int r)
     L.tab_small = 0;
     L.tab_large = nq * 16;
     L.bar_off = 2 * nq * 16;
-    L.buf_off = (L.bar_off + kBoxWarps * 2 * 8 + 127) & ~127;
-    L.total = L.buf_off + kBoxWarps * kBoxBytes;
+    L.buf_off = (L.bar_off + kBoxWarps * 2 * 8 + 127) & ~127;   // TMA destinations: 128-byte aligned
+    L.total = L.buf_off + kBoxWarps * kBoxBytes + 128;   // + alignment slack
     return L;
 }
 

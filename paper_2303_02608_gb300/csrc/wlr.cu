@@ -384,10 +384,11 @@ __global__ void __launch_bounds__(kTilePix, 2)
 // tile-staged kernel over the flagged-tile queue.
 template <bool kMixed>
 __global__ void __launch_bounds__(kTilePix, 2)
-    wlr_adaptive_kernel(const __grid_constant__ CUtensorMap tmap, const WlrParams p)
+    wlr_adaptive_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap box_small,
+                        const __grid_constant__ CUtensorMap box_large, const WlrParams p)
 {
     if (p.sparse_max > 0 && *(volatile uint32_t*)&p.ctrl->flag_total <= p.sparse_max)
-        sparse_body<kSparsePerWarp, kMixed>(p, SingleSeq{&p});
+        sparse_body<kSparsePerWarp, kMixed>(p, SingleSeq{&p, &box_small, &box_large});
     else
         tile_body<false, kMixed>(tmap, p);
 }
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(kSolveThreads, 3) wlr_solve_kernel(const WlrPa
     if (threadIdx.x == 0 && blockIdx.x == 0)
         p.ctrl->ev_base = p.ctrl->ev_total;   // records not yet drained come first
     const uint32_t n = p.dense ? (uint32_t)((size_t)p.W * p.H) : *(volatile uint32_t*)&p.ctrl->list_len;
-    const unsigned long long fp64 = solve_records<kMixed>(p, SingleSeq{&p}, n);
+    const unsigned long long fp64 = solve_records<kMixed>(p, SingleSeq{&p, nullptr, nullptr}, n);
     finish(p, 0ull, 0ull, fp64, false, false);
 }
 
@@ -470,19 +471,18 @@ int wlr_grid(int smem_bytes, int num_sms, bool mixed, bool adaptive)
     return per_sm * num_sms;
 }
 
-cudaError_t launch_wlr(const CUtensorMap& tmap, const WlrParams& p, bool mixed, int grid, int smem_bytes,
-                       cudaStream_t s)
+cudaError_t launch_wlr(const RingMaps& m, const WlrParams& p, bool mixed, int grid, int smem_bytes, cudaStream_t s)
 {
     if (mixed) {
         if (p.dense)
-            wlr_dense_kernel<true><<<grid, kTilePix, smem_bytes, s>>>(tmap, p);
+            wlr_dense_kernel<true><<<grid, kTilePix, smem_bytes, s>>>(m.tile, p);
         else
-            wlr_adaptive_kernel<true><<<grid, kTilePix, smem_bytes, s>>>(tmap, p);
+            wlr_adaptive_kernel<true><<<grid, kTilePix, smem_bytes, s>>>(m.tile, m.box_small, m.box_large, p);
     } else {
         if (p.dense)
-            wlr_dense_kernel<false><<<grid, kTilePix, smem_bytes, s>>>(tmap, p);
+            wlr_dense_kernel<false><<<grid, kTilePix, smem_bytes, s>>>(m.tile, p);
         else
-            wlr_adaptive_kernel<false><<<grid, kTilePix, smem_bytes, s>>>(tmap, p);
+            wlr_adaptive_kernel<false><<<grid, kTilePix, smem_bytes, s>>>(m.tile, m.box_small, m.box_large, p);
     }
     return cudaGetLastError();
 }
