@@ -120,6 +120,9 @@ struct esim_ad_ctx {
     size_t N = 0;
     int tiles_x = 0, tiles_y = 0, n_tiles = 0, n_chunks = 0;
     int smem_bytes = 0;          // dense tile-staged regression
+    int smem_ex = 0;             // exhaustive regression,
+    int ex_group = 1;            // the frames it stages together
+    int ex_grid = 0;
     int smem_adaptive = 0;       // adaptive regression: the larger of its two forms
     int nbuf = 2;
     int wlr_grid = 0;
@@ -295,10 +298,13 @@ esim_ad_status encode_ring_map(esim_ad_ctx* c)
     const cuuint64_t dims[4] = {mixed ? 8u : 4u, (cuuint64_t)c->W, (cuuint64_t)c->H,
                                 (cuuint64_t)((mixed ? 1 : 2) * c->cfg.frames)};
     const cuuint64_t strides[3] = {16, (cuuint64_t)16 * c->W, (cuuint64_t)16 * c->W * c->H};
-    const cuuint32_t box[4] = {mixed ? 8u : 4u, (cuuint32_t)(kTileX + 2 * c->cfg.radius),
-                               (cuuint32_t)(kTileY + 2 * c->cfg.radius), mixed ? 1u : 2u};
-    return encode_tiled(&c->maps.tile, mixed ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
-                        c->ring, dims, strides, box) &&
+    const int halo = 2 * c->cfg.radius;
+    auto encode = [&](CUtensorMap* m, int tx, int ty) {
+        const cuuint32_t box[4] = {mixed ? 8u : 4u, (cuuint32_t)(tx + halo), (cuuint32_t)(ty + halo), mixed ? 1u : 2u};
+        return encode_tiled(m, mixed ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, c->ring,
+                            dims, strides, box);
+    };
+    return encode(&c->maps.tile, kTileX, kTileY) && encode(&c->maps.ex_tile, kExTileX, kExTileY) &&
                    encode_boxes(&c->maps, c->ring, c->W, c->H, c->cfg.frames, mixed)
                ? ESIM_AD_OK
                : ESIM_AD_ECUDA;
@@ -380,8 +386,9 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
     c->tiles_y = (c->H + kTileY - 1) / kTileY;
     c->n_tiles = c->tiles_x * c->tiles_y;
     c->n_chunks = (int)((c->N + kChunk - 1) / kChunk);
-    int max_smem_sm = 0, num_sms = 0;
+    int max_smem_sm = 0, max_smem_block = 0, num_sms = 0;
     if (cudaDeviceGetAttribute(&max_smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&max_smem_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
         delete c;
@@ -459,6 +466,16 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
     c->wlr_grid = wlr_grid(c->smem_bytes, num_sms, c->mixed, false);
     c->adaptive_grid = wlr_grid(c->smem_adaptive, num_sms, c->mixed, true);
     c->solve_grid = wlr_solve_grid(num_sms);
+    if (cfg->mode == ESIM_AD_EXHAUSTIVE) {
+        c->smem_ex = exhaustive_smem(cfg->radius, cfg->frames, c->mixed, max_smem_sm, &c->ex_group);
+        if (exhaustive_prepare(max_smem_block, c->mixed) != cudaSuccess) {
+            cudaGetLastError();
+            release(c);
+            delete c;
+            return ESIM_AD_ECUDA;
+        }
+        c->ex_grid = exhaustive_grid(c->smem_ex, num_sms, c->W, c->H, c->mixed);
+    }
     // staged ingest for FP16/BF16 frames in the precision form (frames of at
     // least one tile); ESIM_AD_INGEST_STAGED=0 keeps the one-tile kernel
     if (c->mixed && cfg->radiance_fmt == ESIM_AD_LOGLUMA_F16 && cfg->feature_fmt == ESIM_AD_FEAT_BF16 &&
@@ -664,6 +681,7 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
     wp.tiles_x = c->tiles_x;
     wp.n_tiles = c->n_tiles;
     wp.nbuf = c->nbuf;
+    wp.frame_group = c->ex_group;
     wp.dense = adaptive_test ? 0 : 1;
     wp.init = c->t == 0 ? 1 : 0;
     wp.sw = kTileX + 2 * c->cfg.radius;
@@ -700,12 +718,17 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
     wp.ctrl = c->ctrl;
     {
         ProfScope ps(c, 1, c->stream);
-        // pass 1: dense frames tile-staged over every tile; adaptive frames in one
-        // launch that picks window boxes or the tile queue from the flagged total
-        const int grid = wp.dense ? (c->n_tiles < c->wlr_grid ? c->n_tiles : c->wlr_grid) : c->adaptive_grid;
-        if (launch_wlr(c->maps, wp, c->mixed, grid, wp.dense ? c->smem_bytes : c->smem_adaptive, c->stream) !=
-            cudaSuccess)
-            return ESIM_AD_ECUDA;
+        // pass 1: exhaustive frames; frame 0 of an adaptive sequence tile-staged over
+        // every tile; adaptive frames in one launch that picks window boxes or the
+        // tile queue from the flagged total
+        cudaError_t e;
+        if (c->cfg.mode == ESIM_AD_EXHAUSTIVE) {
+            e = launch_exhaustive(c->maps.ex_tile, wp, c->mixed, c->ex_grid, c->smem_ex, c->stream);
+        } else {
+            const int grid = wp.dense ? (c->n_tiles < c->wlr_grid ? c->n_tiles : c->wlr_grid) : c->adaptive_grid;
+            e = launch_wlr(c->maps, wp, c->mixed, grid, wp.dense ? c->smem_bytes : c->smem_adaptive, c->stream);
+        }
+        if (e != cudaSuccess) return ESIM_AD_ECUDA;
         // pass 2: solve every accumulated system and emit; it follows the
         // previous frame's event writer (it sets ev_base from that frame's total)
         if (join_writer(c) != cudaSuccess ||

@@ -146,6 +146,7 @@ struct WlrParams {
     int W, H, r, T, t, n_tau, tiles_x, n_tiles;
     int mixed;             // ring in the mixed form (FP16/BF16), refined + FP64-fallback solve
     int nbuf;              // staged frames in flight per CTA (2 or 3)
+    int frame_group;       // exhaustive kernel: frames staged together
     int dense;             // 1: every tile and pixel; 0: tiles from the queue
     int init;              // 1: frame 0 (initialise models, no events)
     int sw, sh;            // staged tile: (32 + 2r) x (8 + 2r) pixels
@@ -217,9 +218,10 @@ int ingest_staged_grid(int sms);
 // Autotuning cache (tune_cache.cu): value for key, or 0 if none.
 int tune_cache_lookup(const char* key);
 void tune_cache_store(const char* key, int value);
-// TMA views of a ring: one box per staged tile, and the window boxes.
+// TMA views of a ring: one box per staged tile (for exhaustive frames the
+// exhaustive kernel's tile), and the window boxes.
 struct RingMaps {
-    CUtensorMap tile, box_small, box_large;
+    CUtensorMap tile, ex_tile, box_small, box_large;
 };
 // Tiled map without swizzle or interleave; out-of-range elements read as zero.
 bool encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t rank, const void* ptr, const cuuint64_t* dims,
@@ -235,6 +237,13 @@ size_t wlr_smem_bytes(int r, bool mixed, int max_smem_per_sm, int* nbuf);
 int wlr_grid(int smem_bytes, int num_sms, bool mixed, bool adaptive);
 int wlr_sparse_smem(int r, bool mixed);
 cudaError_t launch_wlr(const RingMaps& m, const WlrParams& p, bool mixed, int grid, int smem_bytes, cudaStream_t s);
+// Regression pass 1 of exhaustive frames: tiles of 16 x 4 pixels, four lanes per pixel.
+constexpr int kExTileX = 16, kExLanes = 4, kExTileY = kTilePix / kExTileX / kExLanes;
+int exhaustive_smem(int r, int T, bool mixed, int max_smem_per_sm, int* group);
+cudaError_t exhaustive_prepare(int max_smem_block, bool mixed);
+int exhaustive_grid(int smem_bytes, int num_sms, int W, int H, bool mixed);
+cudaError_t launch_exhaustive(const CUtensorMap& tmap, const WlrParams& p, bool mixed, int grid, int smem_bytes,
+                              cudaStream_t s);
 cudaError_t launch_wlr_solve(const WlrParams& p, bool mixed, int grid, cudaStream_t s);
 int wlr_solve_grid(int num_sms);
 cudaError_t launch_events(const EventParams& p, cudaStream_t s);

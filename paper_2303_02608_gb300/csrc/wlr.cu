@@ -1,5 +1,5 @@
 // Weighted local regression (Eqs. 3-5) with event emission (Eq. 1), in two
-// passes per frame.
+// passes per frame (exhaustive frames' first pass is in exhaustive.cu).
 //
 // Pass 1 accumulates.  For every regressed pixel the kernel-weighted sums of
 // the normal equations over the spatio-temporal window (the Gram matrix of
@@ -7,9 +7,10 @@
 // stored as one 272-byte Gram record.  Two forms share this pass:
 //   tile-staged   - a 32x8 pixel tile plus an r-pixel halo of one ring frame
 //                   per stage, landed by one 4-D TMA load, up to three stages in
-//                   flight per persistent CTA; every pixel of every tile (dense
-//                   frames, wlr_dense_kernel) or the flagged pixels of the queued
-//                   tiles (adaptive frames with many flags);
+//                   flight per persistent CTA; every pixel of every tile (frame 0
+//                   of an adaptive sequence, wlr_dense_kernel; exhaustive frames:
+//                   exhaustive.cu) or the flagged pixels of the queued tiles
+//                   (adaptive frames with many flags);
 //   window boxes  - per-warp boxes covering the windows of four flagged pixels,
 //                   landed by bulk asynchronous copies (adaptive frames with few
 //                   flags).
@@ -370,7 +371,7 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
 }
 
 
-// Dense frames (frame 0, exhaustive mode): every tile, tile-staged.
+// Frame 0 of an adaptive sequence: every tile, tile-staged.
 template <bool kMixed>
 __global__ void __launch_bounds__(kTilePix, 2)
     wlr_dense_kernel(const __grid_constant__ CUtensorMap tmap, const WlrParams p)

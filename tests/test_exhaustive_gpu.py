@@ -1,0 +1,36 @@
+"""The exhaustive regression's tiles (16 x 4 pixels, four lanes each) and frame
+groups against the FP64 oracle: whole and partial tiles, windows larger than the
+image, more frames than are staged together.  Tolerance: alpha within 1e-4."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import EXHAUSTIVE, Oracle, OracleConfig
+from scenes import Scene, SceneConfig
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("W,H,r,T,n", [
+    (1, 1, 1, 1, 2),      # one pixel
+    (16, 4, 3, 2, 3),     # exactly one tile
+    (17, 5, 3, 2, 3),     # one pixel past it
+    (40, 21, 7, 5, 7),    # interior and clipped tiles, a full temporal window
+    (23, 9, 15, 3, 4),    # the largest radius: one frame per group
+    (36, 20, 9, 7, 8),    # two groups of frames, of unequal length
+])
+def test_exhaustive_alpha_matches_oracle(W, H, r, T, n):
+    import paper_2303_02608_gb300 as m
+    cfg = SceneConfig(kind="rects", width=W, height=H, frames=n, spp=2, seed=W + r, rgb=True,
+                      n_rects=max(3, W * H // 150), bg_depth=10.0)
+    sim = m.Simulator(m.SimConfig(width=W, height=H, radius=r, frames=T, contrast=0.2, mode=m.ESIM_AD_EXHAUSTIVE))
+    orc = Oracle(OracleConfig(W, H, radius=r, frames=T, channels=3, mode=EXHAUSTIVE, contrast=0.2))
+    for f in Scene(cfg).sequence():
+        sim.push({k: f[k].cuda() for k in ("radiance", "normal", "albedo", "depth")})
+        orc.push({k: f[k].numpy() for k in ("radiance", "normal", "albedo", "depth")})
+        a, flags = sim.denoised()
+        assert np.abs(a.cpu().numpy() - orc.outputs()["alpha"].reshape(H, W)).max() <= 1e-4
+        assert bool(torch.all(flags == 1))
+    stats = sim.stats()
+    assert stats["regressions"] == W * H * n
+    sim.close()
