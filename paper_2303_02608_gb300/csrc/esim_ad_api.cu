@@ -304,6 +304,8 @@ esim_ad_status encode_ring_map(esim_ad_ctx* c)
         return encode_tiled(m, mixed ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, c->ring,
                             dims, strides, box);
     };
+    const int rows = wlr_rows(c->cfg.radius, mixed);
+    if (rows && !encode(&c->maps.rows, kTileX, rows)) return ESIM_AD_ECUDA;
     return encode(&c->maps.tile, kTileX, kTileY) && encode(&c->maps.ex_tile, kExTileX, kExTileY) &&
                    encode_boxes(&c->maps, c->ring, c->W, c->H, c->cfg.frames, mixed)
                ? ESIM_AD_OK
@@ -452,10 +454,7 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
         return ESIM_AD_ECUDA;
     }
     memset(c->marks, 0, sizeof(HostMarks));
-    {
-        const int sp = wlr_sparse_smem(cfg->radius, c->mixed);
-        c->smem_adaptive = c->smem_bytes > sp ? c->smem_bytes : sp;
-    }
+    c->smem_adaptive = wlr_adaptive_smem(cfg->radius, c->mixed, c->smem_bytes);
     if (encode_ring_map(c) != ESIM_AD_OK ||
         wlr_prepare(c->smem_bytes, c->smem_adaptive, c->mixed) != cudaSuccess) {
         cudaGetLastError();

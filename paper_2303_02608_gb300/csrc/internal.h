@@ -221,7 +221,7 @@ void tune_cache_store(const char* key, int value);
 // TMA views of a ring: one box per staged tile (for exhaustive frames the
 // exhaustive kernel's tile), and the window boxes.
 struct RingMaps {
-    CUtensorMap tile, ex_tile, box_small, box_large;
+    CUtensorMap tile, ex_tile, box_small, box_large, rows;
 };
 // Tiled map without swizzle or interleave; out-of-range elements read as zero.
 bool encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t rank, const void* ptr, const cuuint64_t* dims,
@@ -235,7 +235,9 @@ bool encode_boxes(RingMaps* m, const void* ring, int W, int H, int T, bool mixed
 cudaError_t wlr_prepare(int smem_dense, int smem_adaptive, bool mixed);
 size_t wlr_smem_bytes(int r, bool mixed, int max_smem_per_sm, int* nbuf);
 int wlr_grid(int smem_bytes, int num_sms, bool mixed, bool adaptive);
-int wlr_sparse_smem(int r, bool mixed);
+// Tile rows of a row box, 0 where the windows are too wide for one.
+int wlr_rows(int r, bool mixed);
+int wlr_adaptive_smem(int r, bool mixed, int tile_smem);
 cudaError_t launch_wlr(const RingMaps& m, const WlrParams& p, bool mixed, int grid, int smem_bytes, cudaStream_t s);
 // Regression pass 1 of exhaustive frames: tiles of 16 x 4 pixels, four lanes per pixel.
 constexpr int kExTileX = 16, kExLanes = 4, kExTileY = kTilePix / kExTileX / kExLanes;

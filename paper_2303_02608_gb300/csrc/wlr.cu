@@ -75,6 +75,67 @@ __host__ __device__ inline SmemLayout smem_layout(int r, int nbuf, bool mixed)
     return L;
 }
 
+// Sum a lane's share (offsets sub, sub + g, ...) of one frame of a pixel's window, clipped to
+// [dxlo, dxhi] x [dylo, dyhi], from a box of row pitch `sw` in which the pixel lies at (sx, sy).
+template <class At>
+__device__ __forceinline__ void walk_window(const At& at, int g, int sub, int dxlo, int dxhi, int dylo, int dyhi,
+                                            int r, int sx, int sy, int sw, const float4* table, float spx)
+{
+    const int side = 2 * r + 1, nx = dxhi - dxlo + 1, ny = dyhi - dylo + 1;
+    if (g == 1) {
+        for (int oy = dylo; oy <= dyhi; ++oy) {
+            const float u2 = (float)oy * spx;
+            const float en_row = -u2 * u2;
+            const int row = (sy + oy) * sw + sx;
+            float u1 = (float)dxlo * spx;
+            // the mixed form's larger loop body runs faster without unrolling
+#pragma unroll 1
+            for (int ox = dxlo; ox <= dxhi; ++ox) {
+                at(row + ox, u1, u2, fmaf(-u1, u1, en_row));
+                u1 += spx;
+            }
+        }
+    } else if (nx == side && ny == side) {
+        // interior pixel: walk the full window through the table
+        const int cbase = sy * sw + sx;
+        for (int q = sub; q < side * side; q += g) {
+            const float4 e = table[q];
+            at(cbase + __float_as_int(e.w), e.x, e.y, e.z);
+        }
+    } else {
+        // window clipped by the image border
+        const int nvalid = nx * ny;
+        int ox = dxlo + sub % nx;
+        int oy = dylo + sub / nx;
+        for (int q = sub; q < nvalid; q += g) {
+            const int si = (sy + oy) * sw + sx + ox;
+            const float u1 = (float)ox * spx;
+            const float u2 = (float)oy * spx;
+            at(si, u1, u2, -fmaf(u1, u1, u2 * u2));
+            ox += g;
+            while (ox > dxhi) {
+                ox -= nx;
+                ++oy;
+            }
+        }
+    }
+}
+
+// Lanes per pixel (log2) of a work item of npix pixels of one tile.
+__device__ __forceinline__ int queue_lanes(int npix)
+{
+    return npix > 128 ? 0 : npix > 64 ? 1 : npix > 32 ? 2 : npix > 16 ? 3 : npix > 8 ? 4 : 5;
+}
+
+// Pixels per work item of the flagged-tile queue, from the frame's flagged total.
+__device__ __forceinline__ int queue_chunk(uint32_t total)
+{
+    const uint32_t target = total / (uint32_t)(gridDim.x * 8u);
+    int chunk = 16;
+    while (chunk < kTilePix && (uint32_t)chunk < target) chunk <<= 1;
+    return chunk;
+}
+
 // Persistent regression kernel.  Each CTA pulls work items from a counter
 // (every tile in dense mode, chunks of the active-tile queue otherwise) and
 // keeps up to nbuf staged frames in flight, each a (work item, tau) pair
@@ -123,10 +184,7 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
     // chunk w % per); chunks past a tile's count are empty and skipped.
     int chunk = kTilePix, per = 1, n_items = n_work;
     if (!kDense) {
-        const uint32_t total = *(volatile uint32_t*)&p.ctrl->flag_total;
-        const uint32_t target = total / (uint32_t)(gridDim.x * 8u);
-        chunk = 16;
-        while (chunk < kTilePix && (uint32_t)chunk < target) chunk <<= 1;
+        chunk = queue_chunk(*(volatile uint32_t*)&p.ctrl->flag_total);
         per = kTilePix / chunk;
         n_items = n_work * per;
     }
@@ -257,7 +315,7 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
             const int tx0 = (in.tile % p.tiles_x) * kTileX, ty0 = (in.tile / p.tiles_x) * kTileY;
             npix = in.count;
             lg = 0;
-            if (!kDense) lg = npix > 128 ? 0 : npix > 64 ? 1 : npix > 32 ? 2 : npix > 16 ? 3 : npix > 8 ? 4 : 5;
+            if (!kDense) lg = queue_lanes(npix);
             g = 1 << lg;
             const int item = (int)threadIdx.x >> lg;
             sub = (int)threadIdx.x & (g - 1);
@@ -293,47 +351,8 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
                 kc = pair_const(sf, cf);
             }
         }
-        if (active) {
-            const int nx = dxhi - dxlo + 1;
-            if (g == 1) {
-                for (int oy = dylo; oy <= dyhi; ++oy) {
-                    const float u2 = (float)oy * spx;
-                    const float en_row = -u2 * u2;
-                    const int row = (sy + oy) * p.sw + sx;
-                    float u1 = (float)dxlo * spx;
-                    // the mixed form's larger loop body runs faster without unrolling
-                    constexpr int kRowUnroll = 1;
-#pragma unroll kRowUnroll
-                    for (int ox = dxlo; ox <= dxhi; ++ox) {
-                        at(row + ox, u1, u2, fmaf(-u1, u1, en_row));
-                        u1 += spx;
-                    }
-                }
-            } else if (nx == side && dyhi - dylo + 1 == side) {
-                // interior pixel: walk the full window through the table
-                const int cbase = sy * p.sw + sx;
-                for (int q = sub; q < nq; q += g) {
-                    const float4 e = table[q];
-                    at(cbase + __float_as_int(e.w), e.x, e.y, e.z);
-                }
-            } else {
-                // window clipped by the image border
-                const int nvalid = nx * (dyhi - dylo + 1);
-                int ox = dxlo + sub % nx;
-                int oy = dylo + sub / nx;
-                for (int q = sub; q < nvalid; q += g) {
-                    const int si = (sy + oy) * p.sw + sx + ox;
-                    const float u1 = (float)ox * spx;
-                    const float u2 = (float)oy * spx;
-                    at(si, u1, u2, -fmaf(u1, u1, u2 * u2));
-                    ox += g;
-                    while (ox > dxhi) {
-                        ox -= nx;
-                        ++oy;
-                    }
-                }
-            }
-        }
+        if (active)
+            walk_window(at, g, sub, dxlo, dxhi, dylo, dyhi, p.r, sx, sy, p.sw, table, spx);
         // count this warp out of the buffer; the last warp refills it
         __syncwarp();
         if (lane == 0) {
@@ -370,6 +389,173 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
     finish(p, s_pairs, s_pix, 0ull, timed_out || (threadIdx.x == 0 && !pr->ok), false);
 }
 
+// Row boxes of the flagged-tile queue: each warp takes 32 lanes' worth of a
+// work item's pixels (with the lanes per pixel of the tile-staged form, so the
+// sums are the same bit for bit) and stages the tile's width plus halo of the
+// `rows` tile rows that they lie in, one frame at a time.  An item's pixels
+// leave on average a quarter of a CTA's lanes without work, and in the
+// tile-staged form those warps wait for the others; here each goes on to the
+// next unit.  A unit's pixels follow one another in raster order, so they
+// rarely need more rows than a box holds; those that do are done in passes.
+// Four warps per scheduler hide the wait for a copy (1-2 us against the 30-40
+// of summing a frame).
+constexpr int kRowsBytes = 13312;   // per warp; with 8 warps two CTAs fit on an SM
+struct RowsLayout {
+    int rows, bar_off, buf_off, total;
+};
+__host__ __device__ inline RowsLayout rows_layout(int r, bool mixed)
+{
+    RowsLayout L;
+    const int fit = kRowsBytes / ((mixed ? 16 : 32) * (kTileX + 2 * r)) - 2 * r;
+    L.rows = fit < kTileY ? fit : kTileY;
+    L.bar_off = (2 * r + 1) * (2 * r + 1) * 16;
+    L.buf_off = (L.bar_off + kBoxWarps * 8 + 127) & ~127;   // TMA destinations: 128-byte aligned
+    L.total = L.buf_off + kBoxWarps * kRowsBytes + 128;     // + alignment slack
+    return L;
+}
+// A box holds the rows of 32 consecutive pixels of a tile that is half flagged: three, as the
+// run starts anywhere in a row.  Wider windows (r > 7, FP32 r > 3) are staged by tiles.
+__host__ __device__ inline bool rows_fit(int r, bool mixed) { return rows_layout(r, mixed).rows >= 3; }
+
+template <bool kMixed>
+__device__ __forceinline__ void rows_body(const CUtensorMap& rmap, const WlrParams& p)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
+    const RowsLayout L = rows_layout(p.r, kMixed);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4* table = reinterpret_cast<float4*>(smem);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.bar_off) + warp;
+    unsigned char* buf = smem + L.buf_off + warp * kRowsBytes;
+    const int side = 2 * p.r + 1;
+    const int plane = p.sw * (L.rows + 2 * p.r);   // records of a box
+    const uint32_t box_bytes = (uint32_t)((kMixed ? 16 : 32) * plane);
+    const float spx = p.s_coord_px;
+    const float* sf = kMixed ? p.q_scale : p.s_feat;
+    __shared__ unsigned long long s_pairs, s_pix;
+    for (int q = threadIdx.x; q < side * side; q += blockDim.x) {
+        const int ox = q % side - p.r, oy = q / side - p.r;
+        const float u1 = (float)ox * spx, u2 = (float)oy * spx;
+        table[q] = make_float4(u1, u2, -fmaf(u1, u1, u2 * u2), __int_as_float(oy * p.sw + ox));
+    }
+    if (threadIdx.x == 0) {
+        s_pairs = 0ull;
+        s_pix = 0ull;
+    }
+    if (lane == 0) {
+        mbar_init(bar, 1);
+        mbar_fence_init();
+    }
+    __syncthreads();
+    // Unit w: queue slot, chunk of the tile's pixel list, 32 lanes of the chunk.
+    const uint32_t chunk = (uint32_t)queue_chunk(*(volatile uint32_t*)&p.ctrl->flag_total);
+    const uint32_t per = kTilePix / chunk;
+    const uint32_t n_units = *(volatile uint32_t*)&p.ctrl->tile_count * per * kBoxWarps;
+    const float4* P0 = reinterpret_cast<const float4*>(buf);
+    const float4* P1 = P0 + plane;
+    const uint4* PM = reinterpret_cast<const uint4*>(buf);
+    uint32_t phase = 0u;
+    bool timed_out = false;
+    AccP acc;
+    for (;;) {
+        int tile = -1, first = 0, count = 0, unit = 0;
+        if (lane == 0) {
+            for (;;) {
+                const uint32_t w = atomicAdd(&p.ctrl->work_next, 1u);
+                if (w >= n_units) break;
+                const uint32_t item = w / kBoxWarps;
+                const int t = (int)p.tile_queue[item / per];
+                first = (int)(item % per * chunk);
+                count = min((int)chunk, (int)p.tile_nflag[t] - first);
+                unit = (int)(w % kBoxWarps);
+                if (count <= 0) {   // past the tile's pixels: on to the next tile
+                    atomicMax(&p.ctrl->work_next, (item / per + 1u) * per * kBoxWarps);
+                } else if (unit * (32 >> queue_lanes(count)) >= count) {   // to the next item
+                    atomicMax(&p.ctrl->work_next, (item + 1u) * kBoxWarps);
+                } else {
+                    tile = t;
+                    break;
+                }
+            }
+        }
+        tile = __shfl_sync(0xffffffffu, tile, 0);
+        if (tile < 0) break;
+        first = __shfl_sync(0xffffffffu, first, 0);
+        count = __shfl_sync(0xffffffffu, count, 0);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        const int lg = queue_lanes(count), g = 1 << lg, sub = lane & (g - 1);
+        const int idx = unit * (32 >> lg) + (lane >> lg);
+        const bool active = idx < count;
+        const int lidx = active ? (int)p.tile_pix[(size_t)tile * kTilePix + first + idx] : 0;
+        const int lx = lidx & (kTileX - 1), ly = lidx / kTileX;
+        const int tx0 = (tile % p.tiles_x) * kTileX, ty0 = (tile / p.tiles_x) * kTileY;
+        const int cx = tx0 + lx, cy = ty0 + ly;
+        const int dxlo = max(-p.r, -cx), dxhi = min(p.r, p.W - 1 - cx);
+        const int dylo = max(-p.r, -cy), dyhi = min(p.r, p.H - 1 - cy);
+        PairConst kc;
+        accp_zero(acc);
+        bool todo = active;
+        while (!timed_out) {
+            const int y0 = __reduce_min_sync(0xffffffffu, todo ? ly : kTileY);
+            if (y0 == kTileY) break;
+            const bool mine = todo && ly < y0 + L.rows;
+            todo = todo && !mine;
+            const int sx = lx + p.r, sy = ly - y0 + p.r;
+            for (int k = 0; k < p.n_tau; ++k) {
+                // every lane is past its reads of the frame before
+                __syncwarp();
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    const int slot = (p.t - k) % p.T;
+                    mbar_arrive_expect_tx(bar, box_bytes);
+                    tma_load_4d(buf, &rmap, bar, 0, tx0 - p.r, ty0 + y0 - p.r, kMixed ? slot : 2 * slot);
+                }
+                __syncwarp();
+                const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase, p.poll_limit));
+                if (!ok) {
+                    mbar_wait_bounded(bar, phase, p.poll_limit);   // one more chance to land
+                    timed_out = true;
+                    break;
+                }
+                phase ^= 1u;
+                if (!mine) continue;
+                if (k == 0) {
+                    float c[7];
+                    if (kMixed) {
+                        float yc;
+                        unpack_mixed(PM[sy * p.sw + sx], yc, c);
+                    } else {
+                        const float4 c0 = P0[sy * p.sw + sx];
+                        const float4 c1 = P1[sy * p.sw + sx];
+                        c[0] = c0.y; c[1] = c0.z; c[2] = c0.w; c[3] = c1.x; c[4] = c1.y; c[5] = c1.z; c[6] = c1.w;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 7; ++j) c[j] *= sf[j];
+                    kc = pair_const(sf, c);
+                }
+                auto at = [&](int si, float u1, float u2, float en0) {
+                    if (kMixed)
+                        accp(acc, PM[si], make_float2(u1, u2), en0, kc);
+                    else
+                        accp(acc, P0[si], P1[si], make_float2(u1, u2), en0, kc);
+                };
+                walk_window(at, g, sub, dxlo, dxhi, dylo, dyhi, p.r, sx, sy, p.sw, table, spx);
+            }
+        }
+        if (timed_out) break;
+        if (g > 1) accp_reduce(acc, g);
+        if (active) {
+            accp_store(acc, p.gram + (size_t)(p.tile_base[tile] + (uint32_t)(first + idx)) * kGramStride, sub, g);
+            if (sub == 0) {
+                atomicAdd(&s_pairs, (unsigned long long)((dxhi - dxlo + 1) * (dyhi - dylo + 1) * p.n_tau));
+                atomicAdd(&s_pix, 1ull);
+            }
+        }
+    }
+    __syncthreads();
+    finish(p, s_pairs, s_pix, 0ull, timed_out, false);
+}
 
 // Frame 0 of an adaptive sequence: every tile, tile-staged.
 template <bool kMixed>
@@ -386,10 +572,13 @@ __global__ void __launch_bounds__(kTilePix, 2)
 template <bool kMixed>
 __global__ void __launch_bounds__(kTilePix, 2)
     wlr_adaptive_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap box_small,
-                        const __grid_constant__ CUtensorMap box_large, const WlrParams p)
+                        const __grid_constant__ CUtensorMap box_large, const __grid_constant__ CUtensorMap rows,
+                        const WlrParams p)
 {
     if (p.sparse_max > 0 && *(volatile uint32_t*)&p.ctrl->flag_total <= p.sparse_max)
         sparse_body<kSparsePerWarp, kMixed>(p, SingleSeq{&p, &box_small, &box_large});
+    else if (rows_fit(p.r, kMixed))
+        rows_body<kMixed>(rows, p);
     else
         tile_body<false, kMixed>(tmap, p);
 }
@@ -412,7 +601,13 @@ __global__ void __launch_bounds__(kSolveThreads, 3) wlr_solve_kernel(const WlrPa
     finish(p, 0ull, 0ull, fp64, false, false);
 }
 
-int wlr_sparse_smem(int r, bool /*mixed*/) { return box_layout(r).total; }
+int wlr_rows(int r, bool mixed) { return rows_fit(r, mixed) ? rows_layout(r, mixed).rows : 0; }
+
+int wlr_adaptive_smem(int r, bool mixed, int tile_smem)
+{
+    const int boxes = box_layout(r).total, queue = rows_fit(r, mixed) ? rows_layout(r, mixed).total : tile_smem;
+    return boxes > queue ? boxes : queue;
+}
 
 int wlr_solve_grid(int num_sms) { return 3 * num_sms; }   // one wave at 3 CTAs per SM
 
@@ -478,12 +673,12 @@ cudaError_t launch_wlr(const RingMaps& m, const WlrParams& p, bool mixed, int gr
         if (p.dense)
             wlr_dense_kernel<true><<<grid, kTilePix, smem_bytes, s>>>(m.tile, p);
         else
-            wlr_adaptive_kernel<true><<<grid, kTilePix, smem_bytes, s>>>(m.tile, m.box_small, m.box_large, p);
+            wlr_adaptive_kernel<true><<<grid, kTilePix, smem_bytes, s>>>(m.tile, m.box_small, m.box_large, m.rows, p);
     } else {
         if (p.dense)
             wlr_dense_kernel<false><<<grid, kTilePix, smem_bytes, s>>>(m.tile, p);
         else
-            wlr_adaptive_kernel<false><<<grid, kTilePix, smem_bytes, s>>>(m.tile, m.box_small, m.box_large, p);
+            wlr_adaptive_kernel<false><<<grid, kTilePix, smem_bytes, s>>>(m.tile, m.box_small, m.box_large, m.rows, p);
     }
     return cudaGetLastError();
 }
