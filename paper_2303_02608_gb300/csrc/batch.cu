@@ -7,8 +7,8 @@
 //      compacted into one queue of (sequence, pixel) entries (sequence in the
 //      top 8 bits), each tile's run padded to four entries,
 //   4. one persistent accumulation launch over that queue (the single-sequence
-//      window-box form: per-warp boxes of an item's windows landed by bulk
-//      asynchronous copies, packed FP32 sums, one Gram record per entry; the
+//      window-box form: per-warp boxes of an item's windows landed by TMA
+//      box loads, packed FP32 sums, one Gram record per entry; the
 //      item size, hence lanes per pixel, is a template choice),
 //   5. one solve launch over the records (solve, Eq. 1 emission into each
 //      sequence's maps, scan of the per-chunk event counts),

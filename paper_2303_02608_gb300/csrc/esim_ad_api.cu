@@ -120,8 +120,7 @@ struct esim_ad_ctx {
     size_t N = 0;
     int tiles_x = 0, tiles_y = 0, n_tiles = 0, n_chunks = 0;
     int smem_bytes = 0;          // dense tile-staged regression
-    int smem_ex = 0;             // exhaustive regression,
-    int ex_group = 1;            // the frames it stages together
+    int smem_ex = 0;             // exhaustive regression of large windows; 0: tile-staged
     int ex_grid = 0;
     int smem_adaptive = 0;       // adaptive regression: the larger of its two forms
     int nbuf = 2;
@@ -465,8 +464,8 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
     c->wlr_grid = wlr_grid(c->smem_bytes, num_sms, c->mixed, false);
     c->adaptive_grid = wlr_grid(c->smem_adaptive, num_sms, c->mixed, true);
     c->solve_grid = wlr_solve_grid(num_sms);
-    if (cfg->mode == ESIM_AD_EXHAUSTIVE) {
-        c->smem_ex = exhaustive_smem(cfg->radius, cfg->frames, c->mixed, max_smem_sm, &c->ex_group);
+    if (cfg->mode == ESIM_AD_EXHAUSTIVE) c->smem_ex = exhaustive_smem(cfg->radius, cfg->frames, c->mixed, max_smem_sm);
+    if (c->smem_ex) {
         if (exhaustive_prepare(max_smem_block, c->mixed) != cudaSuccess) {
             cudaGetLastError();
             release(c);
@@ -680,7 +679,6 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
     wp.tiles_x = c->tiles_x;
     wp.n_tiles = c->n_tiles;
     wp.nbuf = c->nbuf;
-    wp.frame_group = c->ex_group;
     wp.dense = adaptive_test ? 0 : 1;
     wp.init = c->t == 0 ? 1 : 0;
     wp.sw = kTileX + 2 * c->cfg.radius;
@@ -717,11 +715,11 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
     wp.ctrl = c->ctrl;
     {
         ProfScope ps(c, 1, c->stream);
-        // pass 1: exhaustive frames; frame 0 of an adaptive sequence tile-staged over
-        // every tile; adaptive frames in one launch that picks window boxes or the
+        // pass 1: exhaustive frames of large windows; other exhaustive frames and frame 0
+        // of an adaptive sequence tile-staged over every tile; adaptive frames in one launch that picks window boxes or the
         // tile queue from the flagged total
         cudaError_t e;
-        if (c->cfg.mode == ESIM_AD_EXHAUSTIVE) {
+        if (c->smem_ex) {
             e = launch_exhaustive(c->maps.ex_tile, wp, c->mixed, c->ex_grid, c->smem_ex, c->stream);
         } else {
             const int grid = wp.dense ? (c->n_tiles < c->wlr_grid ? c->n_tiles : c->wlr_grid) : c->adaptive_grid;

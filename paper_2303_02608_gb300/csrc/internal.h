@@ -146,7 +146,6 @@ struct WlrParams {
     int W, H, r, T, t, n_tau, tiles_x, n_tiles;
     int mixed;             // ring in the mixed form (FP16/BF16), refined + FP64-fallback solve
     int nbuf;              // staged frames in flight per CTA (2 or 3)
-    int frame_group;       // exhaustive kernel: frames staged together
     int dense;             // 1: every tile and pixel; 0: tiles from the queue
     int init;              // 1: frame 0 (initialise models, no events)
     int sw, sh;            // staged tile: (32 + 2r) x (8 + 2r) pixels
@@ -239,9 +238,10 @@ int wlr_grid(int smem_bytes, int num_sms, bool mixed, bool adaptive);
 int wlr_rows(int r, bool mixed);
 int wlr_adaptive_smem(int r, bool mixed, int tile_smem);
 cudaError_t launch_wlr(const RingMaps& m, const WlrParams& p, bool mixed, int grid, int smem_bytes, cudaStream_t s);
-// Regression pass 1 of exhaustive frames: tiles of 16 x 4 pixels, four lanes per pixel.
+// Regression pass 1 of exhaustive frames with large windows: tiles of 16 x 4 pixels, four
+// lanes per pixel.  exhaustive_smem is 0 for the windows that the tile-staged kernel keeps.
 constexpr int kExTileX = 16, kExLanes = 4, kExTileY = kTilePix / kExTileX / kExLanes;
-int exhaustive_smem(int r, int T, bool mixed, int max_smem_per_sm, int* group);
+int exhaustive_smem(int r, int T, bool mixed, int max_smem_per_sm);
 cudaError_t exhaustive_prepare(int max_smem_block, bool mixed);
 int exhaustive_grid(int smem_bytes, int num_sms, int W, int H, bool mixed);
 cudaError_t launch_exhaustive(const CUtensorMap& tmap, const WlrParams& p, bool mixed, int grid, int smem_bytes,

@@ -1,5 +1,6 @@
 // Weighted local regression (Eqs. 3-5) with event emission (Eq. 1), in two
-// passes per frame (exhaustive frames' first pass is in exhaustive.cu).
+// passes per frame (the first pass of exhaustive frames with large windows is in
+// exhaustive.cu).
 //
 // Pass 1 accumulates.  For every regressed pixel the kernel-weighted sums of
 // the normal equations over the spatio-temporal window (the Gram matrix of
@@ -8,12 +9,15 @@
 //   tile-staged   - a 32x8 pixel tile plus an r-pixel halo of one ring frame
 //                   per stage, landed by one 4-D TMA load, up to three stages in
 //                   flight per persistent CTA; every pixel of every tile (frame 0
-//                   of an adaptive sequence, wlr_dense_kernel; exhaustive frames:
-//                   exhaustive.cu) or the flagged pixels of the queued tiles
+//                   of an adaptive sequence and exhaustive frames,
+//                   wlr_dense_kernel; large windows: exhaustive.cu) or the
+//                   flagged pixels of the queued tiles (adaptive frames with many
+//                   flags and windows too wide for row boxes);
+//   row boxes     - per-warp boxes of a few rows of a queued tile plus halo
 //                   (adaptive frames with many flags);
-//   window boxes  - per-warp boxes covering the windows of four flagged pixels,
-//                   landed by bulk asynchronous copies (adaptive frames with few
-//                   flags).
+//   window boxes  - per-warp boxes covering the windows of four flagged pixels
+//                   (adaptive frames with few flags); both landed by one TMA load
+//                   per frame.
 // Adaptive frames launch wlr_adaptive_kernel, which picks the form on the
 // device from the frame's flagged total.
 // Each regressed pixel is owned by g lanes (g = 1 when a tile is densely
@@ -398,7 +402,8 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
 // next unit.  A unit's pixels follow one another in raster order, so they
 // rarely need more rows than a box holds; those that do are done in passes.
 // Four warps per scheduler hide the wait for a copy (1-2 us against the 30-40
-// of summing a frame).
+// of summing a frame).  FP32-bound: 1920 x 1080, 500,000 pixels flagged, 15 x 15 x 5
+// window, precision form: 2121 us (53% of the FP32 peak), tile-staged 2543.
 constexpr int kRowsBytes = 13312;   // per warp; with 8 warps two CTAs fit on an SM
 struct RowsLayout {
     int rows, bar_off, buf_off, total;
@@ -557,7 +562,7 @@ __device__ __forceinline__ void rows_body(const CUtensorMap& rmap, const WlrPara
     finish(p, s_pairs, s_pix, 0ull, timed_out, false);
 }
 
-// Frame 0 of an adaptive sequence: every tile, tile-staged.
+// Every tile, tile-staged: frame 0 of an adaptive sequence, exhaustive frames.
 template <bool kMixed>
 __global__ void __launch_bounds__(kTilePix, 2)
     wlr_dense_kernel(const __grid_constant__ CUtensorMap tmap, const WlrParams p)
@@ -567,8 +572,8 @@ __global__ void __launch_bounds__(kTilePix, 2)
 
 // Adaptive frames: one launch that picks its form on the device from the
 // frame's flagged total (known only after the test kernel ran): per-warp
-// window boxes when at most sparse_max pixels are flagged, else the
-// tile-staged kernel over the flagged-tile queue.
+// window boxes when at most sparse_max pixels are flagged, else the flagged-tile
+// queue by row boxes, or tile-staged where the windows are too wide for them.
 template <bool kMixed>
 __global__ void __launch_bounds__(kTilePix, 2)
     wlr_adaptive_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap box_small,

@@ -278,11 +278,10 @@ __device__ __forceinline__ void accp_offset(AccP& a, const OffSums& o, float2 q0
     a.x[0] = fmaf(t.x, q0.y, a.x[0]);
 }
 
-// Butterfly sum over the g lanes (a power of two), kStride apart, that share a pixel.
-template <int kStride = 1>
+// Butterfly sum over the g adjacent lanes (a power of two) that share a pixel.
 __device__ __forceinline__ void accp_reduce(AccP& a, int g)
 {
-    for (int off = kStride * g >> 1; off >= kStride; off >>= 1) {
+    for (int off = g >> 1; off > 0; off >>= 1) {
         a.g0 += __shfl_xor_sync(0xffffffffu, a.g0, off);
         a.s4 += __shfl_xor_sync(0xffffffffu, a.s4, off);
 #pragma unroll

@@ -1,6 +1,7 @@
-"""The exhaustive regression's tiles (16 x 4 pixels, four lanes each) and frame
-groups against the FP64 oracle: whole and partial tiles, windows larger than the
-image, more frames than are staged together.  Tolerance: alpha within 1e-4."""
+"""The exhaustive regression's two forms (tiles of 16 x 4 pixels, four lanes each,
+for large windows; tile-staged otherwise) against the FP64 oracle: whole and
+partial tiles, windows larger than the image.
+Tolerance: alpha within 1e-4."""
 import numpy as np
 import pytest
 import torch
@@ -13,11 +14,12 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("W,H,r,T,n", [
     (1, 1, 1, 1, 2),      # one pixel
+    (1, 1, 7, 5, 2),
+    (16, 4, 7, 5, 6),     # large windows: exactly one tile
+    (17, 5, 8, 5, 6),     # one pixel past it
     (16, 4, 3, 2, 3),     # exactly one tile
     (17, 5, 3, 2, 3),     # one pixel past it
     (40, 21, 7, 5, 7),    # interior and clipped tiles, a full temporal window
-    (23, 9, 15, 3, 4),    # the largest radius: one frame per group
-    (36, 20, 9, 7, 8),    # two groups of frames, of unequal length
 ])
 def test_exhaustive_alpha_matches_oracle(W, H, r, T, n):
     import paper_2303_02608_gb300 as m
