@@ -56,6 +56,9 @@ FP32_LANES_PER_SM = 128
 # the equilibration of the 1596 Gram entries (3192 + 55 rsqrt) and the
 # Cholesky of the augmented 56 x 56 system (2 x 55 x 56 x 57 / 6 = 58520
 # trailing-update flop, 1540 column scalings, 55 sqrt, 2 for alpha) -> 63472.
+# This counts the method's normal equations.  The kernel accumulates their 770
+# distinct sums only, so its own FP32 work per pair is about half of it, and the
+# fraction of peak reported at this count is not one of pipe occupancy.
 FLOP_PER_NEIGHBOUR_2 = 3326
 FLOP_PER_SOLVE_2 = 63472
 
@@ -940,8 +943,9 @@ def _quality(dev, C_values=(0.25, 0.5, 0.75, 1.0), taus=(5e-4, 1e-3, 2e-3, 5e-3,
 # accumulation is the simulator's (162); bwd_center_kernel re-forms the
 # regressors (14), the squared distance (17), exp2 (1), the fit and v'^T u
 # (18 each), dalpha/dw (3), its weight (2) and the seven bandwidth terms (21) =
-# 94; bwd_source_kernel the regressors, distance, exp2, v'^T u and one FMA =
-# 52.  Per centre the forward solve for theta' and v' (ridge, equilibration,
+# 94; a source's sum over its centres the regressors, distance, exp2, v'^T u and
+# one FMA = 52 (bwd_source_kernel; at this window the centre pass yields those
+# sums too and forms the pair's weight once).  Per centre the forward solve for theta' and v' (ridge, equilibration,
 # Cholesky, two substitution pairs): about 900.
 FLOP_FWD_PAIR, FLOP_BWD_CENTER_PAIR, FLOP_BWD_SOURCE_PAIR, FLOP_FWD_SOLVE = 162, 94, 52, 900
 
