@@ -130,6 +130,7 @@ struct esim_ad_ctx {
     int sparse_stage = 1;        // sparse kernel stages window boxes (ESIM_AD_SPARSE_STAGE=0: L1 only)
     int test_withhold = 0;       // ESIM_AD_TEST_WITHHOLD_COPY=1: timeout injection for tests
     bool mixed = false;
+    uint32_t rows_min = 0;       // the others with at least this many take row boxes where their windows fit them
     uint32_t sparse_max = 0;     // adaptive frames with at most this many flagged pixels use the sparse kernel
     float4* ring = nullptr;
     float4* state = nullptr;
@@ -497,6 +498,12 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
     if (const char* e = getenv("ESIM_AD_SPARSE_MAX")) {
         if (*e) c->sparse_max = (uint32_t)strtoul(e, nullptr, 10);
     }
+    // of the other frames, those with enough flagged pixels for whole tiles as work
+    // items take row boxes (the same results); ESIM_AD_ROWS_MIN overrides the line
+    c->rows_min = wlr_rows_min(c->adaptive_grid);
+    if (const char* e = getenv("ESIM_AD_ROWS_MIN")) {
+        if (*e) c->rows_min = (uint32_t)strtoul(e, nullptr, 10);
+    }
     if (const char* e = getenv("ESIM_AD_SPARSE_STAGE")) {
         if (*e == '0') c->sparse_stage = 0;
     }
@@ -705,6 +712,7 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
     wp.n_chunks = c->n_chunks;
     wp.emit_events = c->t > 0 ? 1 : 0;
     wp.sparse_max = c->sparse_max;
+    wp.rows_min = c->rows_min;
     wp.flag_list = c->flag_list;
     wp.sparse_stage = c->sparse_stage;
     wp.tile_base = c->tile_base;

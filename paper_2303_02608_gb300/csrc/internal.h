@@ -167,6 +167,7 @@ struct WlrParams {
     unsigned long long* chunk_off;   // exclusive offsets, written by the last CTA
     int n_chunks;
     int emit_events;                 // 0 on frame 0 (no events)
+    uint32_t rows_min;               // queue mode: from this many flagged pixels on -> row boxes
     uint32_t sparse_max;             // queue mode: at most this many flagged pixels -> sparse kernel
     const uint32_t* flag_list;       // flagged pixel indices per tile, each run padded to 4 entries
     int sparse_stage;                // sparse kernel: 1 stage window boxes in shared memory, 0 read via L1
@@ -237,6 +238,7 @@ int wlr_grid(int smem_bytes, int num_sms, bool mixed, bool adaptive);
 // Tile rows of a row box, 0 where the windows are too wide for one.
 int wlr_rows(int r, bool mixed);
 int wlr_adaptive_smem(int r, bool mixed, int tile_smem);
+uint32_t wlr_rows_min(int grid);
 cudaError_t launch_wlr(const RingMaps& m, const WlrParams& p, bool mixed, int grid, int smem_bytes, cudaStream_t s);
 // Regression pass 1 of exhaustive frames with large windows: tiles of 16 x 4 pixels, four
 // lanes per pixel.  exhaustive_smem is 0 for the windows that the tile-staged kernel keeps.

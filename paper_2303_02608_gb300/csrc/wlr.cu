@@ -12,9 +12,9 @@
 //                   of an adaptive sequence and exhaustive frames,
 //                   wlr_dense_kernel; large windows: exhaustive.cu) or the
 //                   flagged pixels of the queued tiles (adaptive frames with many
-//                   flags and windows too wide for row boxes);
+//                   flags);
 //   row boxes     - per-warp boxes of a few rows of a queued tile plus halo
-//                   (adaptive frames with many flags);
+//                   (adaptive frames with very many flags);
 //   window boxes  - per-warp boxes covering the windows of four flagged pixels
 //                   (adaptive frames with few flags); both landed by one TMA load
 //                   per frame.
@@ -404,6 +404,11 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
 // Four warps per scheduler hide the wait for a copy (1-2 us against the 30-40
 // of summing a frame).  FP32-bound: 1920 x 1080, 500,000 pixels flagged, 15 x 15 x 5
 // window, precision form: 2121 us (53% of the FP32 peak), tile-staged 2543.
+// Taken when work items are whole tiles (rows_min, the total from which
+// queue_chunk gives 256).  Below that an item has many lanes per pixel and little
+// to sum per frame, and a warp's one box in flight shows: frames of 480 x 300, 7 x 7 x 3
+// window, took 195 us against 153 tile-staged, 15 x 15 x 5 327 against 308; of
+// 1500 x 1000, above it, 404 against 457 and 1623 against 1924.
 constexpr int kRowsBytes = 13312;   // per warp; with 8 warps two CTAs fit on an SM
 struct RowsLayout {
     int rows, bar_off, buf_off, total;
@@ -573,7 +578,8 @@ __global__ void __launch_bounds__(kTilePix, 2)
 // Adaptive frames: one launch that picks its form on the device from the
 // frame's flagged total (known only after the test kernel ran): per-warp
 // window boxes when at most sparse_max pixels are flagged, else the flagged-tile
-// queue by row boxes, or tile-staged where the windows are too wide for them.
+// queue by row boxes (at least rows_min flagged pixels, windows that fit them) or
+// tile-staged.
 template <bool kMixed>
 __global__ void __launch_bounds__(kTilePix, 2)
     wlr_adaptive_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap box_small,
@@ -582,7 +588,7 @@ __global__ void __launch_bounds__(kTilePix, 2)
 {
     if (p.sparse_max > 0 && *(volatile uint32_t*)&p.ctrl->flag_total <= p.sparse_max)
         sparse_body<kSparsePerWarp, kMixed>(p, SingleSeq{&p, &box_small, &box_large});
-    else if (rows_fit(p.r, kMixed))
+    else if (rows_fit(p.r, kMixed) && *(volatile uint32_t*)&p.ctrl->flag_total >= p.rows_min)
         rows_body<kMixed>(rows, p);
     else
         tile_body<false, kMixed>(tmap, p);
@@ -608,10 +614,14 @@ __global__ void __launch_bounds__(kSolveThreads, 3) wlr_solve_kernel(const WlrPa
 
 int wlr_rows(int r, bool mixed) { return rows_fit(r, mixed) ? rows_layout(r, mixed).rows : 0; }
 
+uint32_t wlr_rows_min(int grid) { return (uint32_t)grid * 8u * (kTilePix / 2) + 1u; }
+
 int wlr_adaptive_smem(int r, bool mixed, int tile_smem)
 {
-    const int boxes = box_layout(r).total, queue = rows_fit(r, mixed) ? rows_layout(r, mixed).total : tile_smem;
-    return boxes > queue ? boxes : queue;
+    int total = box_layout(r).total;
+    if (tile_smem > total) total = tile_smem;
+    if (rows_fit(r, mixed) && rows_layout(r, mixed).total > total) total = rows_layout(r, mixed).total;
+    return total;
 }
 
 int wlr_solve_grid(int num_sms) { return 3 * num_sms; }   // one wave at 3 CTAs per SM

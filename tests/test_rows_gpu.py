@@ -35,16 +35,18 @@ def _mask(kind, rng):
 
 def _alpha(frames, r, T, precision, path):
     import paper_2303_02608_gb300 as m
-    old = os.environ.pop("ESIM_AD_SPARSE_MAX", None)
-    os.environ["ESIM_AD_SPARSE_MAX"] = path
+    keys = {"ESIM_AD_SPARSE_MAX": path, "ESIM_AD_ROWS_MIN": "0"}
+    old = {k: os.environ.pop(k, None) for k in keys}
+    os.environ.update(keys)
     try:
         sim = m.Simulator(m.SimConfig(width=W, height=H, radius=r, frames=T, contrast=0.5, mode=m.ESIM_AD_ADAPTIVE,
                                       radiance_fmt=m.ESIM_AD_LOGLUMA_F16, feature_fmt=m.ESIM_AD_FEAT_F32,
                                       precision=precision, guard_kappa=1.0))
     finally:
-        os.environ.pop("ESIM_AD_SPARSE_MAX", None)
-        if old is not None:
-            os.environ["ESIM_AD_SPARSE_MAX"] = old
+        for k in keys:
+            os.environ.pop(k, None)
+            if old[k] is not None:
+                os.environ[k] = old[k]
     for f in frames:
         sim.push({k: v.cuda() for k, v in f.items()})
     a, flags = sim.denoised()
