@@ -18,6 +18,7 @@
 // its own ring, model state and maps, exactly as a single-sequence context
 // does; the per-pixel arithmetic is shared with it.
 #include <errno.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <sys/stat.h>
 #include <stdlib.h>
@@ -55,6 +56,7 @@ struct SeqStep {
 struct BatchGlobal {
     const SeqStep* steps;
     const RingMaps* maps;        // TMA views of each sequence's ring
+    int n_seq;
     const uint16_t* tile_seq;    // global tile -> sequence
     const uint16_t* chunk_seq;   // global chunk -> sequence
     uint32_t* flag_list;         // (seq << 24) | pixel
@@ -67,6 +69,10 @@ struct BatchGlobal {
     float s_px;
     Ctrl* ctrl;
 };
+
+static_assert(sizeof(RingMaps) % 128 == 0 && offsetof(RingMaps, box_small) % 128 == 0 &&
+                  offsetof(RingMaps, box_large) % 128 == 0,
+              "tensor maps in global memory: 128-byte aligned, from an aligned allocation on");
 
 // Tile shapes the autotuner chooses from: width in pixels (height 256 / width).
 constexpr int kTileShapes = 3;
@@ -128,10 +134,17 @@ __global__ void __launch_bounds__(kTilePix) batch_ingest_kernel(BatchGlobal g)
 
 // Pass 1: one persistent launch over the queue of every sequence, in the
 // single-sequence window-box form (items of kItem entries; an item stays
-// inside one tile of one sequence).
+// inside one tile of one sequence).  The rings' tensor maps lie in global memory,
+// written by the host when the batch was made, perhaps where an earlier batch's
+// lay: each block acquires them before its first load (sparse_body's first
+// barrier orders the fences before every warp's loads).
 template <int kItem, bool kMixed>
 __global__ void __launch_bounds__(kTilePix, 2) batch_wlr_kernel(BatchGlobal g, const WlrParams gp)
 {
+    for (int i = threadIdx.x; i < g.n_seq; i += kTilePix) {
+        fence_tensormap_acquire_sys(&g.maps[i].box_small);
+        if (kMixed) fence_tensormap_acquire_sys(&g.maps[i].box_large);
+    }
     sparse_body<kItem, kMixed>(gp, BatchSeq{g.steps, g.maps});
 }
 
@@ -325,6 +338,7 @@ BatchGlobal globals(const esim_ad_batch* b, int shape)
     BatchGlobal g;
     g.steps = b->d_steps;
     g.maps = b->d_maps;
+    g.n_seq = b->n;
     g.tile_seq = b->tile_seq_s[shape];
     g.chunk_seq = b->chunk_seq;
     g.flag_list = b->flag_list;

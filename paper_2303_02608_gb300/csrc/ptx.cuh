@@ -99,6 +99,16 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
         : "memory");
 }
 
+// Order this thread block's later TMA accesses through the tensor map at `map`
+// (global memory, 128-byte aligned) after the host's write of it.  Needed once
+// per block for a map in global memory, whose address may have held another one
+// before; kernel parameters (__grid_constant__) need none.
+__device__ __forceinline__ void fence_tensormap_acquire_sys(const CUtensorMap* map)
+{
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(map))
+                 : "memory");
+}
+
 // 2^x on the MUFU unit (ex2.approx, flush-to-zero).
 __device__ __forceinline__ float ex2_approx(float x)
 {

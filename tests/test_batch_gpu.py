@@ -135,3 +135,41 @@ def test_batch_benchmark_window_with_1080p_member(pair, tmp_path):
     reps, stats = _run(ADAPTIVE, pair, tmp_path, shapes=shapes, spans=spans, n_steps=7, r=7, t_win=5, c=0.15,
                        bands=bands, spp=2)
     assert all(r["regressed"] > 0 for r in reps) and sum(r["events"] for r in reps) > 0
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_batches_made_in_turn_read_their_own_rings(mixed):
+    """Batches of different sizes made and destroyed in turn, so that one's device
+    structures take the place of another's: each sequence against a context of
+    its own on the same frames, the flagged pixels chosen by a brightness step
+    under the variance guard.  Either form is within 1e-4 of the FP64 oracle, so
+    the two lie within 2e-4 of one another."""
+    import paper_2303_02608_gb300 as m
+    for turn in range(6):
+        shapes = [[(96, 72), (40, 30)], [(33, 60), (130, 20), (64, 64)]][turn % 2]
+        cfgs = [m.SimConfig(width=w, height=h, radius=3, frames=2, contrast=0.5, guard_kappa=1.0,
+                            radiance_fmt=m.ESIM_AD_LOGLUMA_F16, feature_fmt=m.ESIM_AD_FEAT_F32,
+                            precision=m.ESIM_AD_MIXED if mixed else m.ESIM_AD_FP32) for w, h in shapes]
+        seqs, masks = [], []
+        for i, (w, h) in enumerate(shapes):
+            rng = np.random.default_rng(10 * turn + i)
+            mask = torch.from_numpy(rng.random((h, w)) < 0.1)
+            feat = torch.from_numpy(rng.uniform(-1, 1, (7, h, w)).astype(np.float32)).cuda()
+            noise = torch.from_numpy(rng.normal(0.0, 0.01, (3, h, w)).astype(np.float32))
+            seqs.append([{"radiance": (noise[t] + 2.0 * (t == 2) * mask).half().cuda(),
+                          "variance": torch.zeros(h, w, device="cuda"), "normal": feat[:3].contiguous(),
+                          "depth": feat[3].contiguous(), "albedo": feat[4:].contiguous()} for t in range(3)])
+            masks.append(mask.numpy())
+        batch = m.Batch(cfgs)
+        for t in range(3):
+            batch.step([s[t] for s in seqs])
+        got = [[v.cpu().numpy() for v in batch.denoised(i)] for i in range(len(shapes))]
+        batch.close()
+        for cfg, frames, mask, (alpha, flags) in zip(cfgs, seqs, masks, got):
+            sim = m.Simulator(cfg)
+            for f in frames:
+                sim.push(f)
+            ref, ref_flags = (v.cpu().numpy() for v in sim.denoised())
+            sim.close()
+            assert np.array_equal(flags != 0, mask) and np.array_equal(flags, ref_flags)
+            assert np.abs(alpha - ref).max() <= 2e-4
