@@ -163,3 +163,33 @@ def test_full_size_sequence_sampled():
     err = np.abs(alpha.numpy()[:, 250:254] - ref[:, 250:254]).max()
     assert err <= 1e-4, err
     assert np.isfinite(loss) and torch.isfinite(g_rad).all() and torch.isfinite(g_b).all()
+
+
+def test_infinite_share_of_the_bandwidth_gradient():
+    """A centre tile's share of the gradient that exceeds FP32's range leaves the
+    gradient infinite with its sign.  Rows of equal pixels make the 32 centres of
+    one row of the middle tile contribute the same, so that scaling the loss by
+    a power of two takes their sum past the range and no summand near it (each
+    at most 2^124).  Scaling is exact but for underflows at the smaller scale."""
+    from paper_2303_02608_gb300 import wlr
+    rng = np.random.default_rng(6)
+    rows = torch.from_numpy(rng.uniform(0.0, 1.0, (8, 24)).astype(np.float32)).cuda()
+    rad = torch.exp(20.0 * (rows[0] - 0.5)).view(1, 1, 24, 1).expand(1, 1, 24, 96).contiguous()
+    feat = (2.0 * rows[1:]).view(1, 7, 24, 1).expand(1, 7, 24, 96).contiguous()
+    g = torch.zeros(1, 24, 96, device="cuda")
+    g[0, 12, 32:64] = 1.0
+
+    def grad(scale):
+        bd = torch.ones(7, device="cuda", requires_grad=True)
+        alpha = wlr(rad, feat, bd, radius=7, frames=1)
+        return torch.autograd.grad(alpha, bd, g * scale)[0].cpu().numpy().astype(np.float64)
+
+    one = grad(1.0)
+    shares = np.abs(one) * 0.5 * np.log2(np.e)          # dL/db = sum of shares / (k^2 b), k^2 = log2(e) / 2
+    scale = 2.0 ** np.floor(124 - np.log2(shares.max() / 32))
+    got, want = grad(scale), one * scale
+    over = shares * scale >= 2.0 ** 128
+    assert over.any() and not np.isnan(got).any()
+    np.testing.assert_array_equal(got[over], np.sign(want[over]) * np.inf)
+    fits = np.abs(want) < 0.99 * float(np.finfo(np.float32).max)
+    np.testing.assert_allclose(got[fits], want[fits], rtol=1e-4)
