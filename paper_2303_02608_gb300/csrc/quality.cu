@@ -229,7 +229,9 @@ __device__ __forceinline__ float nearest2(const QualParams& p, int s, int pol, i
                     const float dx = (float)(j0 + i) * p.invW;
                     const G m = min(l[i], r[i]);
                     const float dy = m == kNoEvent<G> ? INFINITY : (float)m * p.invH;
-                    best = fminf(best, fmaf(dx, dx, dt2) + dy * dy);
+                    // dy^2 is rounded by itself: contracted into the sum, distances that equal
+                    // a threshold would fall on its other side
+                    best = fminf(best, __fadd_rn(fmaf(dx, dx, dt2), __fmul_rn(dy, dy)));
                 }
             }
         }

@@ -123,6 +123,18 @@ def test_quality_column_pass_edges(shape, density):
     _compare(gen, ref)
 
 
+@pytest.mark.parametrize("dx,dy,tau", [(7, 12, 0.025), (14, 24, 0.05)])
+def test_quality_distance_equal_to_the_threshold(dx, dy, tau):
+    """Two events exactly tau apart (1000 x 500: (7/1000)^2 + (12/500)^2 = 0.025^2) are
+    not within tau, as in exact arithmetic; a little more, and they are."""
+    import paper_2303_02608_gb300 as m
+    gen, ref = (torch.zeros(1, 500, 1000, dtype=torch.int32, device="cuda") for _ in range(2))
+    gen[0, 100, 100] = 1
+    ref[0, 100 + dy, 100 + dx] = 2
+    q = m.quality(gen, ref, (tau, 1.001 * tau))
+    assert list(q["precision"]) == [0.0, 1.0] and list(q["recall"]) == [0.0, 1.0]
+
+
 def test_quality_degenerate_sets():
     shape = (5, 8, 8)
     z = np.zeros(shape, np.int64)
