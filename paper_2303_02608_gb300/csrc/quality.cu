@@ -54,6 +54,7 @@ __global__ void esim_frame_kernel(const float* __restrict__ rad, int channels, f
 
 constexpr int kColumns = 32;             // image columns of a column-pass block
 constexpr int kMaxRows = 4096;           // rows whose event masks that block holds
+constexpr int kRowChunkBytes = 16 * kColumns;   // masks and carried rows of 32 rows, both polarities
 constexpr int kQueryThreads = 128;
 constexpr int kQueryPix = 32 * kQueryThreads;   // pixels of a query block
 
@@ -449,9 +450,10 @@ extern "C" esim_ad_status esim_ad_quality(const int32_t* gen, const int32_t* ref
     const bool masks = height <= kMaxRows;
     if (masks) {
         // an image up to kMaxRows high keeps its masks in shared memory, and its distances fit 16 bits
-        const int smem = (height + 31) / 32 * kColumns * 16;
-        if (smem > 48 * 1024 &&
-            cudaFuncSetAttribute(column_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+        const int smem = (height + 31) / 32 * kRowChunkBytes;
+        // the limit that every call needs at most: it is the process's, and other threads set it too
+        if (smem > 48 * 1024 && cudaFuncSetAttribute(column_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     kMaxRows / 32 * kRowChunkBytes) != cudaSuccess)
             return ESIM_AD_ECUDA;
         column_mask_kernel<<<dim3((width + kColumns - 1) / kColumns, frames, 2), kQThreads, smem, s>>>(p);
     } else {

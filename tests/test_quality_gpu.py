@@ -135,6 +135,31 @@ def test_quality_distance_equal_to_the_threshold(dx, dy, tau):
     assert list(q["precision"]) == [0.0, 1.0] and list(q["recall"]) == [0.0, 1.0]
 
 
+def test_quality_from_threads_with_images_of_different_heights():
+    """Evaluations of tall images that need different amounts of shared memory, from
+    several threads at once: none is refused, and all agree."""
+    import threading
+    import paper_2303_02608_gb300 as m
+    errors, results = [], {}
+
+    def work(height, calls):
+        sets = torch.zeros(2, 1, height, 4, dtype=torch.int32, device="cuda")
+        sets[0, 0, 5, 1] = sets[1, 0, height - 7, 2] = 1
+        try:
+            for _ in range(calls):
+                q = m.quality(sets[0], sets[1], (0.5, 2.0))
+                results.setdefault(height, set()).add((tuple(q["precision"]), tuple(q["recall"]), q["chamfer"]))
+        except Exception as e:   # noqa: BLE001 - reported below
+            errors.append((height, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(h, 4000)) for h in (4096, 3200, 3300, 4096)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors and all(len(r) == 1 for r in results.values())
+
+
 def test_quality_degenerate_sets():
     shape = (5, 8, 8)
     z = np.zeros(shape, np.int64)
