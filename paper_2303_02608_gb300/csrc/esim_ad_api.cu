@@ -456,7 +456,7 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
     memset(c->marks, 0, sizeof(HostMarks));
     c->smem_adaptive = wlr_adaptive_smem(cfg->radius, c->mixed, c->smem_bytes);
     if (encode_ring_map(c) != ESIM_AD_OK ||
-        wlr_prepare(c->smem_bytes, c->smem_adaptive, c->mixed) != cudaSuccess) {
+        wlr_prepare(max_smem_block, c->mixed) != cudaSuccess) {
         cudaGetLastError();
         release(c);
         delete c;

@@ -215,13 +215,8 @@ int exhaustive_smem(int r, int T, bool mixed, int max_smem_per_sm)
 
 cudaError_t exhaustive_prepare(int max_smem_block, bool mixed)
 {
-    // the device's limit, not this context's need: contexts of other radii launch the same kernel
-    const void* k = mixed ? (const void*)exhaustive_kernel<true> : (const void*)exhaustive_kernel<false>;
-    cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, k);
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   max_smem_block - (int)a.sharedSizeBytes);
+    return allow_dynamic_smem(mixed ? (const void*)exhaustive_kernel<true> : (const void*)exhaustive_kernel<false>,
+                              max_smem_block);
 }
 
 int exhaustive_grid(int smem_bytes, int num_sms, int W, int H, bool mixed)

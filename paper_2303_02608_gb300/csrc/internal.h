@@ -215,6 +215,10 @@ cudaError_t launch_ingest_staged(const CUtensorMap& map_y, const CUtensorMap& ma
                                  const IngestParams& p, int grid, cudaStream_t s);
 int ingest_staged_grid(int sms);
 
+// Let `kernel` launch with all the dynamic shared memory that a block may have.  The limit is
+// the process's, not a context's: one set to a context's own need would refuse the launches of
+// a context that needs more.
+cudaError_t allow_dynamic_smem(const void* kernel, int max_smem_block);
 // Autotuning cache (tune_cache.cu): value for key, or 0 if none.
 int tune_cache_lookup(const char* key);
 void tune_cache_store(const char* key, int value);
@@ -232,7 +236,7 @@ bool encode_boxes(RingMaps* m, const void* ring, int W, int H, int T, bool mixed
 // choosing on the device between the sparse window-box form and the
 // tile-staged queue form); the adaptive kernel's shared memory is the larger
 // of the two forms'.
-cudaError_t wlr_prepare(int smem_dense, int smem_adaptive, bool mixed);
+cudaError_t wlr_prepare(int max_smem_block, bool mixed);
 size_t wlr_smem_bytes(int r, bool mixed, int max_smem_per_sm, int* nbuf);
 int wlr_grid(int smem_bytes, int num_sms, bool mixed, bool adaptive);
 // Tile rows of a row box, 0 where the windows are too wide for one.

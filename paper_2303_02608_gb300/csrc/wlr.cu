@@ -650,19 +650,21 @@ size_t wlr_smem_bytes(int r, bool mixed, int max_smem_per_sm, int* nbuf)
     return (size_t)L.total;
 }
 
-template <bool kMixed>
-static cudaError_t prepare_one(int smem_dense, int smem_adaptive)
+cudaError_t allow_dynamic_smem(const void* kernel, int max_smem_block)
 {
-    cudaError_t e = cudaFuncSetAttribute(wlr_dense_kernel<kMixed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem_dense);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(wlr_adaptive_kernel<kMixed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                smem_adaptive);
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   max_smem_block - (int)a.sharedSizeBytes);
 }
 
-cudaError_t wlr_prepare(int smem_dense, int smem_adaptive, bool mixed)
+cudaError_t wlr_prepare(int max_smem_block, bool mixed)
 {
-    return mixed ? prepare_one<true>(smem_dense, smem_adaptive) : prepare_one<false>(smem_dense, smem_adaptive);
+    const void* dense = mixed ? (const void*)wlr_dense_kernel<true> : (const void*)wlr_dense_kernel<false>;
+    const void* adaptive = mixed ? (const void*)wlr_adaptive_kernel<true> : (const void*)wlr_adaptive_kernel<false>;
+    const cudaError_t e = allow_dynamic_smem(dense, max_smem_block);
+    return e != cudaSuccess ? e : allow_dynamic_smem(adaptive, max_smem_block);
 }
 
 int wlr_grid(int smem_bytes, int num_sms, bool mixed, bool adaptive)
