@@ -677,9 +677,11 @@ esim_ad_status esim_ad_batch_init(const esim_ad_config* cfgs, int32_t n_seq, voi
         return fail(ESIM_AD_ECUDA);
     // the accumulation kernels' dynamic shared memory: window tables and per-warp boxes
     b->smem = box_layout(b->cfg[0].radius).total;
+    int max_smem_block = 0;
+    if (cudaDeviceGetAttribute(&max_smem_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return fail(ESIM_AD_ECUDA);
     for (int lanes : {8, 16, 32})
-        if (cudaFuncSetAttribute(pick_kernel(lanes, b->mixed), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 b->smem) != cudaSuccess)
+        if (allow_dynamic_smem((const void*)pick_kernel(lanes, b->mixed), max_smem_block) != cudaSuccess)
             return fail(ESIM_AD_ECUDA);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pick_kernel(16, b->mixed), kTilePix, b->smem) !=

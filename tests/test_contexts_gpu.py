@@ -60,3 +60,25 @@ def test_simulators_of_different_radii_in_turn(radii, mixed):
             sim.reset()
     for sim in sims:
         sim.close()
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("radii", [(7, 3), (3, 15, 1)])
+def test_batches_of_different_radii_in_turn(radii, mixed):
+    import paper_2303_02608_gb300 as m
+    frames = _frames(4, mixed)
+
+    def step(batch, f):
+        batch.step([f, f])
+        return batch.denoised(1)
+
+    alone = []
+    for r in radii:
+        batch = m.Batch([_config(m, r, mixed)] * 2)
+        alone.append([step(batch, f) for f in frames])
+        batch.close()
+    batches = [m.Batch([_config(m, r, mixed)] * 2) for r in radii]
+    runs = list(zip(*[[step(batch, f) for batch in batches] for f in frames]))
+    for batch, run, ref in zip(batches, runs, alone):
+        _agree(run, ref)
+        batch.close()
