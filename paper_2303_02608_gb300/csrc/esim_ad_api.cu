@@ -507,11 +507,12 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
     if (const char* e = getenv("ESIM_AD_SPARSE_STAGE")) {
         if (*e == '0') c->sparse_stage = 0;
     }
-    // Timeout injection for tests: ESIM_AD_TEST_WITHHOLD_COPY=1 makes every
-    // warp of the sparse regression kernel skip issuing its first window-box
-    // copy (nothing is in flight for that barrier) and bounds each mbarrier
-    // wait to 64 polls, so the wait gives up, the kernel records the timeout
-    // and returns; the normal bound is unchanged otherwise.
+    // Timeout injection for tests: with ESIM_AD_TEST_WITHHOLD_COPY=1, from the
+    // second frame on, every warp of the sparse regression and every CTA of the
+    // exhaustive one skips issuing its first copy (nothing is in flight for that
+    // barrier) and each mbarrier wait is bounded to 64 polls, so the wait gives
+    // up, the kernel records the timeout and returns; the normal bound is
+    // unchanged otherwise.
     if (const char* e = getenv("ESIM_AD_TEST_WITHHOLD_COPY")) {
         if (*e == '1') c->test_withhold = 1;
     }
@@ -717,8 +718,8 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
     wp.sparse_stage = c->sparse_stage;
     wp.tile_base = c->tile_base;
     wp.gram = c->gram;
-    wp.poll_limit = c->test_withhold ? 64u : kPollLimit;
-    wp.withhold_copy = c->test_withhold;
+    wp.withhold_copy = c->test_withhold && c->t > 0 ? 1 : 0;
+    wp.poll_limit = wp.withhold_copy ? 64u : kPollLimit;
     wp.ev_mask = c->ev_mask + (size_t)par * c->n_chunks * (kChunk / 32);
     wp.ctrl = c->ctrl;
     {

@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kTilePix, 2)
         s_pairs = 0ull;
         s_pix = 0ull;
         s_next[1] = (int)atomicAdd(&p.ctrl->work_next, 1u);
-        if (s_next[1] < n_items) issue(s_next[1]);
+        if (s_next[1] < n_items && !p.withhold_copy) issue(s_next[1]);   // withheld (test): the phase never completes
     }
     __syncthreads();
     int item = s_next[1], par = 0;
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kTilePix, 2)
         const int cx = tx0 + lx, cy = ty0 + ly;
         const bool interior = tx0 >= p.r && ty0 >= p.r && tx0 + kExTileX + p.r <= p.W && ty0 + kTH + p.r <= p.H;
         accp_zero(acc);
-        const bool ok = mbar_wait_bounded(&full, phase);
+        const bool ok = mbar_wait_bounded(&full, phase, p.poll_limit);
         phase ^= 1u;
         if (threadIdx.x == 0) s_next[par] = (int)atomicAdd(&p.ctrl->work_next, 1u);
         if (ok) {
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kTilePix, 2)
         par ^= 1;   // a slow warp may still read the other slot
     }
     // a copy that did not land in time gets one more bounded wait before the CTA exits
-    if (timed_out) mbar_wait_bounded(&full, phase ^ 1u, 1u << 20);
+    if (timed_out) mbar_wait_bounded(&full, phase ^ 1u, p.poll_limit);
     __syncthreads();
     finish(p, s_pairs, s_pix, 0ull, timed_out, false);
 }
