@@ -508,8 +508,8 @@ esim_ad_status esim_ad_init(const esim_ad_config* cfg, void* cuda_stream, esim_a
         if (*e == '0') c->sparse_stage = 0;
     }
     // Timeout injection for tests: with ESIM_AD_TEST_WITHHOLD_COPY=1, from the
-    // second frame on, every warp of the sparse regression and every CTA of the
-    // exhaustive one skips issuing its first copy (nothing is in flight for that
+    // second frame on, every warp of the window-box and row-box forms and every CTA
+    // of the exhaustive one skips issuing its first copy (nothing is in flight for that
     // barrier) and each mbarrier wait is bounded to 64 polls, so the wait gives
     // up, the kernel records the timeout and returns; the normal bound is
     // unchanged otherwise.

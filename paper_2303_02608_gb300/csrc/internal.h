@@ -175,7 +175,7 @@ struct WlrParams {
     float* gram;                     // Gram records [entries][68]: entry = pixel index (dense) or
                                      // position in flag_list (adaptive frames)
     uint32_t poll_limit;             // bound on each mbarrier wait (polls; the tile-staged form has its own)
-    int withhold_copy;               // test only: a warp's first box, or an exhaustive CTA's first tile, is never copied
+    int withhold_copy;               // test only: a warp's first box (window, row), or an exhaustive CTA's first tile, is never copied
     uint32_t* ev_mask = nullptr;     // bit per pixel, set where the pixel emits (nullptr: none kept)
     Ctrl* ctrl;
 };

@@ -516,7 +516,7 @@ __device__ __forceinline__ void rows_body(const CUtensorMap& rmap, const WlrPara
                 __syncwarp();
                 fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0) {
+                if (lane == 0 && !p.withhold_copy) {   // withheld (test): nothing is in flight when the wait gives up
                     const int slot = (p.t - k) % p.T;
                     mbar_arrive_expect_tx(bar, box_bytes);
                     tma_load_4d(buf, &rmap, bar, 0, tx0 - p.r, ty0 + y0 - p.r, kMixed ? slot : 2 * slot);

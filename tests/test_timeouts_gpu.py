@@ -12,7 +12,7 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-def _run(config, env, rgb=True):
+def _run(config, env):
     import paper_2303_02608_gb300 as m
     env = {"ESIM_AD_TEST_WITHHOLD_COPY": "1", **env}
     old = {k: os.environ.get(k) for k in env}
@@ -49,3 +49,10 @@ def _run(config, env, rgb=True):
 @pytest.mark.parametrize("w,h", [(16, 4), (64, 48), (333, 251)])   # one tile, fewer tiles than CTAs, more
 def test_exhaustive_large_windows(w, h):
     _run(lambda m: m.SimConfig(width=w, height=h, radius=7, frames=5, contrast=0.05, mode=m.ESIM_AD_EXHAUSTIVE), {})
+
+
+@pytest.mark.parametrize("mixed,r", [(False, 3), (True, 7)])
+def test_row_boxes(mixed, r):
+    _run(lambda m: m.SimConfig(width=101, height=45, radius=r, frames=3, contrast=0.05,
+                               precision=m.ESIM_AD_MIXED if mixed else m.ESIM_AD_FP32),
+         {"ESIM_AD_SPARSE_MAX": "0", "ESIM_AD_ROWS_MIN": "0"})
