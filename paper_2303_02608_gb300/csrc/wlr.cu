@@ -132,13 +132,17 @@ __device__ __forceinline__ int queue_lanes(int npix)
 }
 
 // Pixels per work item of the flagged-tile queue, from the frame's flagged total.
-__device__ __forceinline__ int queue_chunk(uint32_t total)
+__host__ __device__ constexpr int queue_chunk(uint32_t total, uint32_t grid)
 {
-    const uint32_t target = total / (uint32_t)(gridDim.x * 8u);
+    const uint32_t target = total / (grid * 8u);
     int chunk = 16;
     while (chunk < kTilePix && (uint32_t)chunk < target) chunk <<= 1;
     return chunk;
 }
+// The total from which items are whole tiles.
+constexpr uint32_t whole_tile_total(uint32_t grid) { return grid * 8u * (kTilePix / 2 + 1); }
+static_assert(queue_chunk(whole_tile_total(304), 304) == kTilePix && queue_chunk(whole_tile_total(304) - 1, 304) < kTilePix,
+              "row boxes start where items are whole tiles");
 
 // Persistent regression kernel.  Each CTA pulls work items from a counter
 // (every tile in dense mode, chunks of the active-tile queue otherwise) and
@@ -188,7 +192,7 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
     // chunk w % per); chunks past a tile's count are empty and skipped.
     int chunk = kTilePix, per = 1, n_items = n_work;
     if (!kDense) {
-        chunk = queue_chunk(*(volatile uint32_t*)&p.ctrl->flag_total);
+        chunk = queue_chunk(*(volatile uint32_t*)&p.ctrl->flag_total, gridDim.x);
         per = kTilePix / chunk;
         n_items = n_work * per;
     }
@@ -458,7 +462,7 @@ __device__ __forceinline__ void rows_body(const CUtensorMap& rmap, const WlrPara
     }
     __syncthreads();
     // Unit w: queue slot, chunk of the tile's pixel list, 32 lanes of the chunk.
-    const uint32_t chunk = (uint32_t)queue_chunk(*(volatile uint32_t*)&p.ctrl->flag_total);
+    const uint32_t chunk = (uint32_t)queue_chunk(*(volatile uint32_t*)&p.ctrl->flag_total, gridDim.x);
     const uint32_t per = kTilePix / chunk;
     const uint32_t n_units = *(volatile uint32_t*)&p.ctrl->tile_count * per * kBoxWarps;
     const float4* P0 = reinterpret_cast<const float4*>(buf);
@@ -614,7 +618,7 @@ __global__ void __launch_bounds__(kSolveThreads, 3) wlr_solve_kernel(const WlrPa
 
 int wlr_rows(int r, bool mixed) { return rows_fit(r, mixed) ? rows_layout(r, mixed).rows : 0; }
 
-uint32_t wlr_rows_min(int grid) { return (uint32_t)grid * 8u * (kTilePix / 2) + 1u; }
+uint32_t wlr_rows_min(int grid) { return whole_tile_total((uint32_t)grid); }
 
 int wlr_adaptive_smem(int r, bool mixed, int tile_smem)
 {
