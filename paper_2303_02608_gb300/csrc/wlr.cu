@@ -428,8 +428,13 @@ __host__ __device__ inline RowsLayout rows_layout(int r, bool mixed)
     return L;
 }
 // A box holds the rows of 32 consecutive pixels of a tile that is half flagged: three, as the
-// run starts anywhere in a row.  Wider windows (r > 7, FP32 r > 3) are staged by tiles.
-__host__ __device__ inline bool rows_fit(int r, bool mixed) { return rows_layout(r, mixed).rows >= 3; }
+// run starts anywhere in a row.  Wider windows (r > 7, FP32 r > 3) are staged by tiles, and so
+// are FP32 windows of r < 3: their sums are too short for copying a box per warp, with twice
+// the bytes of the precision form.  Whole frames in us, tile-staged -> row boxes, 1920 x 1080
+// with 350,000 / 620,000 / 1,870,000 flagged pixels: FP32, r = 1, 2 frames 243 -> 276, 317 ->
+// 353, 614 -> 624; r = 2, 3 frames 314 -> 371, 430 -> 476, 803 -> 845; r = 3, 3 frames 417 -> 393,
+// 599 -> 546, 1218 -> 1194; precision form, r = 1, 2 frames 251 -> 235, 333 -> 310, 664 -> 632.
+__host__ __device__ inline bool rows_fit(int r, bool mixed) { return rows_layout(r, mixed).rows >= 3 && (mixed || r >= 3); }
 
 template <bool kMixed>
 __device__ __forceinline__ void rows_body(const CUtensorMap& rmap, const WlrParams& p)

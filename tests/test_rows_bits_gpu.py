@@ -94,27 +94,36 @@ def test_row_boxes_give_the_bits_of_the_tile_staged_form(r, T, mixed, total):
         assert np.array_equal(tiles[2], o[2]) and tiles[3:] == o[3:]
 
 
-@pytest.mark.parametrize("below", [0, 1])
-def test_row_boxes_start_where_work_items_are_whole_tiles(below):
-    """The default line: an item holds a power of two of pixels, at least the
-    flagged total over 8 items per CTA (two CTAs per SM), so it is a whole tile of
-    256 pixels from 129 per item on.  Which form ran shows in a run whose row
-    boxes are never copied: it reports a timeout, the tile-staged form does not."""
+def _form(total, r, mixed):
+    """Which form takes a frame of `total` flagged pixels by default: a run whose
+    row boxes are never copied reports a timeout, the tile-staged form does not."""
     import paper_2303_02608_gb300 as m
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    total = 2 * sms * 8 * 129 - below
     mask = torch.zeros(H * W, dtype=torch.bool)
     mask[torch.randperm(H * W, generator=torch.Generator().manual_seed(1))[:total]] = True
-    mask = mask.view(H, W)
-    sim = _simulator(m, 7, 2, True, {"ESIM_AD_TEST_WITHHOLD_COPY": "1"})
+    sim = _simulator(m, r, 2, mixed, {"ESIM_AD_TEST_WITHHOLD_COPY": "1"})
     try:
-        for f in _frames(mask):
+        for f in _frames(mask.view(H, W)):
             sim.push(f)
-        if below:
-            assert torch.equal(sim.denoised()[1].cpu() != 0, mask)
-        else:
-            with pytest.raises(m.EsimError) as e:
-                sim.denoised()
-            assert e.value.status == m.ESIM_AD_ETIMEOUT
+        assert torch.equal(sim.denoised()[1].cpu() != 0, mask.view(H, W))
+        return "tiles"
+    except m.EsimError as e:
+        assert e.status == m.ESIM_AD_ETIMEOUT
+        return "rows"
     finally:
         sim.close()
+
+
+def _whole_tiles():
+    """The total from which a work item is a whole tile: it holds a power of two of pixels,
+    at least the flagged total over 8 items per CTA, two CTAs per SM."""
+    return 2 * torch.cuda.get_device_properties(0).multi_processor_count * 8 * 129
+
+
+def test_row_boxes_start_where_work_items_are_whole_tiles():
+    assert _form(_whole_tiles(), 7, True) == "rows" and _form(_whole_tiles() - 1, 7, True) == "tiles"
+
+
+@pytest.mark.parametrize("r,mixed,form", [(1, True, "rows"), (7, True, "rows"), (8, True, "tiles"), (1, False, "tiles"),
+                                          (2, False, "tiles"), (3, False, "rows"), (4, False, "tiles")])
+def test_windows_that_row_boxes_take(r, mixed, form):
+    assert _form(_whole_tiles() + 5000, r, mixed) == form
