@@ -18,8 +18,8 @@
 // gradient of a pixel is a sum over the centres whose windows contain it: each
 // centre tile sums its own centres' shares per neighbour (bwd_center_kernel),
 // and bwd_gather_kernel adds the tiles; for windows whose tile sums exceed the
-// workspace, bwd_source_kernel gathers over the centres instead.  Every sum has
-// a fixed order, so every result is deterministic.
+// workspace, bwd_center_gv_kernel and bwd_source_kernel gather over the centres
+// instead.  Every sum has a fixed order, so every result is deterministic.
 #include "esim_ad.h"
 #include "internal.h"
 #include "wlr_math.cuh"
@@ -277,6 +277,27 @@ __global__ void __launch_bounds__(kFwdThreads, 4) fwd_kernel(AdjParams p)
     }
 }
 
+constexpr int kCtrRows = 2;
+constexpr int kCtrThreads = kTilePix / kCtrRows;
+constexpr int kCtrWarps = kCtrThreads / 32;
+
+// A block's share of the bandwidth gradient: tree sum in a fixed order -> one partial per block.
+__device__ __forceinline__ void store_partial(const AdjParams& p, const float (&gb)[7])
+{
+    __shared__ float red[kCtrThreads][8];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) red[threadIdx.x][j] = gb[j];
+    __syncthreads();
+    for (int s = kCtrThreads / 2; s > 0; s >>= 1) {
+        if ((int)threadIdx.x < s)
+#pragma unroll
+            for (int j = 0; j < 7; ++j) red[threadIdx.x][j] += red[threadIdx.x + s][j];
+        __syncthreads();
+    }
+    if (threadIdx.x < 7)
+        p.partials[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 8 + threadIdx.x] = red[0][threadIdx.x];
+}
+
 // Per centre: its share of the bandwidth gradient (sum over its window of
 // g_alpha (d alpha/d w_i) w_i u_ij^2), and g_alpha v'^T u_i w_i, its share of its
 // neighbours' dL/dy.  Each thread takes two centres stacked in one column, so
@@ -286,23 +307,17 @@ __global__ void __launch_bounds__(kFwdThreads, 4) fwd_kernel(AdjParams p)
 // sums, and so are centres that the loss leaves out.
 // A 128-thread CTA covers one 32 x 8 tile.
 //
-// kFused: at each offset the lanes' shares go to neighbouring columns of one row;
+// At each offset the lanes' shares go to neighbouring columns of one row;
 // a rotation by the offset brings them to the lane of their column (what
 // wraps around belongs to the halo on the other side).  A warp's rows are
 // summed in registers over the offsets, the tile's warps in shared memory in
-// warp order, one frame of the window at a time.  Otherwise g_alpha v' is left
-// for bwd_source_kernel, which forms every pair's weight again.
+// warp order, one frame of the window at a time.
 //
 // 512 x 512 x 16, 7 x 7 x 3 window: 1.80 ms and 0.13 ms for the gather, against
 // 1.51 ms and 1.08 ms for bwd_source_kernel (1.93 without loading a record ahead).
-constexpr int kCtrRows = 2;
-constexpr int kCtrThreads = kTilePix / kCtrRows;
-constexpr int kCtrWarps = kCtrThreads / 32;
-
-template <bool kFused>
 __global__ void __launch_bounds__(kCtrThreads, 4) bwd_center_kernel(AdjParams p)
 {
-    extern __shared__ float s_rows[];   // kFused: [frame parity][warp][2r + 2][32 + 2r]
+    extern __shared__ float s_rows[];   // [frame parity][warp][2r + 2][32 + 2r]
     const size_t N = (size_t)p.W * p.H;
     const int f = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -332,13 +347,6 @@ __global__ void __launch_bounds__(kCtrThreads, 4) bwd_center_kernel(AdjParams p)
                 t0[k][i] = sv[(size_t)i * N];
                 v0[k][i] = sv[(size_t)(NZ + i) * N];
             }
-        }
-        if (!kFused) {
-            float4* g = p.gv + (size_t)f * 3 * N + ci;
-            const float a = ga[k];
-            g[0] = make_float4(a * v0[k][0], a * v0[k][1], a * v0[k][2], a * v0[k][3]);
-            g[N] = make_float4(a * v0[k][4], a * v0[k][5], a * v0[k][6], a * v0[k][7]);
-            g[2 * N] = make_float4(a * v0[k][8], a * v0[k][9], 0.0f, 0.0f);
         }
         // lambda v^T P theta in natural units
         float vpt = (s_c * s_c) * (v0[k][1] * t0[k][1] + v0[k][2] * t0[k][2]);
@@ -414,55 +422,144 @@ __global__ void __launch_bounds__(kCtrThreads, 4) bwd_center_kernel(AdjParams p)
                         }
 #pragma unroll
                         for (int j = 0; j < 7; ++j) gb[j] = __ffma2_rn(__fmul2_rn(c, u[j]), u[j], gb[j]);
-                        if (kFused) share = sh.x + sh.y;
+                        share = sh.x + sh.y;
                     }
-                    if (kFused) {
-                        const float got = __shfl_sync(0xffffffffu, share, (lane - ox) & 31);
-                        const bool inside = (unsigned)(lane - ox) < 32u;
-                        main_sum += inside ? got : 0.0f;
-                        halo_sum += inside ? 0.0f : got;
-                    }
+                    const float got = __shfl_sync(0xffffffffu, share, (lane - ox) & 31);
+                    const bool inside = (unsigned)(lane - ox) < 32u;
+                    main_sum += inside ? got : 0.0f;
+                    halo_sum += inside ? 0.0f : got;
                 }
             }
-            if (kFused) {
-                float* out = buf + (warp * rows + k) * span;
-                out[p.r + lane] = main_sum;
-                if (lane < p.r) out[p.r + kTileX + lane] = halo_sum;             // from offsets > 0
-                if (lane >= kTileX - p.r) out[lane - (kTileX - p.r)] = halo_sum;   // from offsets < 0 (r <= 15)
-            }
+            float* out = buf + (warp * rows + k) * span;
+            out[p.r + lane] = main_sum;
+            if (lane < p.r) out[p.r + kTileX + lane] = halo_sum;             // from offsets > 0
+            if (lane >= kTileX - p.r) out[lane - (kTileX - p.r)] = halo_sum;   // from offsets < 0 (r <= 15)
         }
-        if (kFused) {
-            __syncthreads();
-            const int trows = kTileY + 2 * p.r;
-            float* out = p.part + (((size_t)f * gridDim.x + blockIdx.x) * p.T + (f - tau)) * trows * span;
-            for (int i = threadIdx.x; i < trows * span; i += kCtrThreads) {
-                const int R = i / span, col = i - R * span;
-                if (ty0 - p.r + R < 0 || ty0 - p.r + R >= p.H) continue;   // no such source row
-                float sum = 0.0f;
-#pragma unroll
-                for (int w = 0; w < kCtrWarps; ++w) {
-                    const int k = R - kCtrRows * w;
-                    if (k >= 0 && k < rows) sum += buf[(w * rows + k) * span + col];
-                }
-                out[i] = sum;
-            }
-            // the next frame's rows go to the other half: no warp is two barriers behind
-            buf = buf == s_rows ? s_rows + kCtrWarps * rows * span : s_rows;
-        }
-    }
-    // block tree sum in a fixed order -> one partial per block
-    __shared__ float red[kCtrThreads][8];
-#pragma unroll
-    for (int j = 0; j < 7; ++j) red[threadIdx.x][j] = gb[j].x + gb[j].y;
-    __syncthreads();
-    for (int s = kCtrThreads / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
-#pragma unroll
-            for (int j = 0; j < 7; ++j) red[threadIdx.x][j] += red[threadIdx.x + s][j];
         __syncthreads();
+        const int trows = kTileY + 2 * p.r;
+        float* out = p.part + (((size_t)f * gridDim.x + blockIdx.x) * p.T + (f - tau)) * trows * span;
+        for (int i = threadIdx.x; i < trows * span; i += kCtrThreads) {
+            const int R = i / span, col = i - R * span;
+            if (ty0 - p.r + R < 0 || ty0 - p.r + R >= p.H) continue;   // no such source row
+            float sum = 0.0f;
+#pragma unroll
+            for (int w = 0; w < kCtrWarps; ++w) {
+                const int k = R - kCtrRows * w;
+                if (k >= 0 && k < rows) sum += buf[(w * rows + k) * span + col];
+            }
+            out[i] = sum;
+        }
+        // the next frame's rows go to the other half: no warp is two barriers behind
+        buf = buf == s_rows ? s_rows + kCtrWarps * rows * span : s_rows;
     }
-    if (threadIdx.x < 7)
-        p.partials[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 8 + threadIdx.x] = red[0][threadIdx.x];
+    const float share[7] = {gb[0].x + gb[0].y, gb[1].x + gb[1].y, gb[2].x + gb[2].y, gb[3].x + gb[3].y,
+                            gb[4].x + gb[4].y, gb[5].x + gb[5].y, gb[6].x + gb[6].y};
+    store_partial(p, share);
+}
+
+// The same for windows whose tile sums exceed the workspace: g_alpha v' is left for
+// bwd_source_kernel, which forms every pair's weight again.  The centres one by one
+// in single FMAs, out-of-image neighbours not visited.  In packed pairs, as above,
+// without shares to pass on: 512 x 512 x 4, 19 x 19 x 3 window 2.20 ms for 1.97; 24 x 20 x 2,
+// 31 x 31 x 1 window 116 us for 83.
+__global__ void __launch_bounds__(kCtrThreads, 4) bwd_center_gv_kernel(AdjParams p)
+{
+    const size_t N = (size_t)p.W * p.H;
+    const int f = blockIdx.y;
+    const int cx = (blockIdx.x % p.tiles_x) * kTileX + (threadIdx.x & 31);
+    const int cy0 = (blockIdx.x / p.tiles_x) * kTileY + kCtrRows * (threadIdx.x >> 5);
+    float sf[7], s_c, s_px;
+    scales(p, sf, s_c, s_px);
+    float gb[7] = {0, 0, 0, 0, 0, 0, 0};
+    float ga[kCtrRows], lvpt[kCtrRows], th[kCtrRows][NZ], v[kCtrRows][NZ], cf[kCtrRows][7];
+    bool active[kCtrRows];
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < kCtrRows; ++k) {
+        const int cy = cy0 + k;
+        active[k] = false;
+        ga[k] = 0.0f;
+        lvpt[k] = 0.0f;
+#pragma unroll
+        for (int i = 0; i < NZ; ++i) th[k][i] = v[k][i] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 7; ++j) cf[k][j] = 0.0f;
+        if (cx >= p.W || cy >= p.H) continue;
+        const size_t ci = (size_t)cy * p.W + cx;
+        ga[k] = p.g_alpha[(size_t)f * N + ci];
+        const float* sv = p.saved + (size_t)f * 20 * N + ci;
+#pragma unroll
+        for (int i = 0; i < NZ; ++i) {
+            th[k][i] = sv[(size_t)i * N];
+            v[k][i] = sv[(size_t)(NZ + i) * N];
+        }
+        // a centre that the loss leaves out adds nothing, whatever was solved there
+        auto times_ga = [&](float x) { return ga[k] != 0.0f ? ga[k] * x : 0.0f; };
+        float4* g = p.gv + (size_t)f * 3 * N + ci;
+        g[0] = make_float4(times_ga(v[k][0]), times_ga(v[k][1]), times_ga(v[k][2]), times_ga(v[k][3]));
+        g[N] = make_float4(times_ga(v[k][4]), times_ga(v[k][5]), times_ga(v[k][6]), times_ga(v[k][7]));
+        g[2 * N] = make_float4(times_ga(v[k][8]), times_ga(v[k][9]), 0.0f, 0.0f);
+        if (ga[k] == 0.0f) continue;
+        // lambda v^T P theta in natural units
+        float vpt = (s_c * s_c) * (v[k][1] * th[k][1] + v[k][2] * th[k][2]);
+#pragma unroll
+        for (int j = 0; j < 7; ++j) vpt = fmaf(sf[j] * sf[j], v[k][3 + j] * th[k][3 + j], vpt);
+        lvpt[k] = p.ridge * vpt;
+        const float4 c0 = p.packed[(size_t)f * 2 * N + ci];
+        const float4 c1 = p.packed[((size_t)f * 2 + 1) * N + ci];
+        cf[k][0] = c0.y * sf[0];
+        cf[k][1] = c0.z * sf[1];
+        cf[k][2] = c0.w * sf[2];
+        cf[k][3] = c1.x * sf[3];
+        cf[k][4] = c1.y * sf[4];
+        cf[k][5] = c1.z * sf[5];
+        cf[k][6] = c1.w * sf[6];
+        active[k] = true;
+        any = true;
+    }
+    if (any) {
+        // neighbours (cx + ox, ny) inside the image, in the window of some centre row
+        const int dxlo = max(-p.r, -cx), dxhi = min(p.r, p.W - 1 - cx);
+        const int nylo = max(0, cy0 - p.r), nyhi = min(p.H - 1, cy0 + kCtrRows - 1 + p.r);
+        for (int tau = max(0, f - p.T + 1); tau <= f; ++tau) {
+            const float4* P0 = p.packed + (size_t)tau * 2 * N;
+            const float4* P1 = P0 + N;
+            for (int ny = nylo; ny <= nyhi; ++ny) {
+                for (int ox = dxlo; ox <= dxhi; ++ox) {
+                    const float u1 = (float)ox * s_px;
+                    const size_t ni = (size_t)ny * p.W + cx + ox;
+                    const float4 h0 = __ldg(P0 + ni), h1 = __ldg(P1 + ni);
+                    const float fv[7] = {h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+#pragma unroll
+                    for (int k = 0; k < kCtrRows; ++k) {
+                        const int oy = ny - (cy0 + k);
+                        if (!active[k] || oy < -p.r || oy > p.r) continue;
+                        const float u2 = (float)oy * s_px;
+                        float u[7];
+                        float en = -fmaf(u1, u1, u2 * u2);
+#pragma unroll
+                        for (int j = 0; j < 7; ++j) {
+                            u[j] = fmaf(fv[j], sf[j], -cf[k][j]);
+                            en = fmaf(-u[j], u[j], en);
+                        }
+                        const float w = ex2_approx(en);
+                        float fit = th[k][0] + th[k][1] * u1 + th[k][2] * u2;
+                        float vz = v[k][0] + v[k][1] * u1 + v[k][2] * u2;
+#pragma unroll
+                        for (int j = 0; j < 7; ++j) {
+                            fit = fmaf(th[k][3 + j], u[j], fit);
+                            vz = fmaf(v[k][3 + j], u[j], vz);
+                        }
+                        const float dadw = fmaf(vz, h0.x - fit, -lvpt[k]);
+                        const float c = ga[k] * dadw * w;
+#pragma unroll
+                        for (int j = 0; j < 7; ++j) gb[j] = fmaf(c, u[j] * u[j], gb[j]);
+                    }
+                }
+            }
+        }
+    }
+    store_partial(p, gb);
 }
 
 // dL/dE of a pixel from its dL/dy.
@@ -717,12 +814,12 @@ extern "C" esim_ad_status esim_ad_wlr_backward(const esim_ad_wlr_desc* d, const 
     const dim3 grid(L.n_tiles, d->sequence);
     if (L.fused) {
         const int smem = 2 * kCtrWarps * (kCtrRows + 2 * d->radius) * (kTileX + 2 * d->radius) * (int)sizeof(float);
-        if (smem > 40 * 1024 && cudaFuncSetAttribute(bwd_center_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (smem > 40 * 1024 && cudaFuncSetAttribute(bwd_center_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      64 * 1024) != cudaSuccess)
             return ESIM_AD_ECUDA;
-        bwd_center_kernel<true><<<grid, kCtrThreads, smem, s>>>(p);
+        bwd_center_kernel<<<grid, kCtrThreads, smem, s>>>(p);
     } else {
-        bwd_center_kernel<false><<<grid, kCtrThreads, 0, s>>>(p);
+        bwd_center_gv_kernel<<<grid, kCtrThreads, 0, s>>>(p);
     }
     bwd_bandwidth_kernel<<<7, kTilePix, 0, s>>>(p, L.n_blocks);
     if (L.fused) {

@@ -142,6 +142,18 @@ def test_masked_centres_add_nothing():
     assert torch.isfinite(rd.grad[:, :, :, 17:]).all() and not rd.grad[0, :, :, 4:10].any()
 
 
+def test_masked_centres_add_nothing_in_wide_windows():
+    """The same where the tile sums do not fit the workspace."""
+    from paper_2303_02608_gb300 import wlr
+    rad, feat, _ = _crop(RECTS, 20, 30, 60, 16, 3)
+    rad[0, :, 0, 0] = float("nan")
+    rd = rad.cuda().requires_grad_(True)
+    bd = torch.tensor(B, dtype=torch.float32, device="cuda", requires_grad=True)
+    wlr(rd, feat.cuda(), bd, radius=9, frames=3)[0, :, 40:].sum().backward()
+    assert torch.isfinite(bd.grad).all()
+    assert torch.isfinite(rd.grad[0, :, :, 31:]).all() and not rd.grad[0, :, :, 10:31].any()
+
+
 def test_backward_is_deterministic():
     rad, feat, clean = _crop(RECTS, 0, 0, 64, 48, 4)
     a = _gpu(rad, feat, clean, B)
