@@ -36,3 +36,14 @@ def test_exhaustive_alpha_matches_oracle(W, H, r, T, n):
     stats = sim.stats()
     assert stats["regressions"] == W * H * n
     sim.close()
+
+
+@pytest.mark.parametrize("W,H,r,T,n", [
+    (5, 40, 7, 5, 6),     # narrower than the window
+    (40, 5, 7, 5, 6),     # lower
+    (3, 17, 8, 5, 6),     # both
+    (8, 8, 7, 6, 7),      # every offset of the window reaches some pixel
+    (7, 9, 7, 5, 6),      # all but the outermost columns
+])
+def test_exhaustive_images_smaller_than_the_window(W, H, r, T, n):
+    test_exhaustive_alpha_matches_oracle(W, H, r, T, n)
