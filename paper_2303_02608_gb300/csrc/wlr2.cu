@@ -52,7 +52,8 @@
 // Measured at 512 x 512 x 16, 7 x 7 x 3 window: 46.7 ms (55.7 with single FMAs,
 // blocks of 7 and a wholly left-looking order), against 92.0 ms with the
 // Gram accumulated as 36 7 x 7 register tiles (1764 sums per neighbour) and
-// factored in registers, 36 threads per pixel.
+// factored in registers, 36 threads per pixel.  Small inputs stay with that one
+// (wlr2_gram.cu).
 #include <stdlib.h>
 
 #include <utility>
@@ -60,6 +61,7 @@
 #include "esim_ad.h"
 #include "internal.h"
 #include "ptx.cuh"
+#include "wlr2.cuh"
 
 namespace esim {
 namespace {
@@ -75,22 +77,6 @@ constexpr int kPart = 128;                 // neighbour pairs per partial sum
 // Table entries of a neighbour: v_0..v_7, v_0..v_6 again, z, w z^0..w z^4, w y z^0..w y z^2.
 constexpr int kZ = 15, kWz = 16, kWyz = 21, kEntries = 24;
 constexpr int kSegMax = 33, kSegFlush = 16;   // neighbour pairs per table, without and with flushed sums
-
-constexpr float kExp2Scale = 0.84932180028801904272f;  // sqrt(log2(e) / 2)
-
-// Quadratic unknown q (0..44) -> feature pair (a, b), a <= b, a-major order.
-__host__ __device__ constexpr int pair_a(int q)
-{
-    int a = 0;
-    while (q >= 9 - a) { q -= 9 - a; ++a; }
-    return a;
-}
-__host__ __device__ constexpr int pair_b(int q)
-{
-    int a = 0;
-    while (q >= 9 - a) { q -= 9 - a; ++a; }
-    return a + q;
-}
 
 // ------------------------------------------------------- compile-time tables
 
@@ -266,20 +252,6 @@ __host__ __device__ constexpr Places places()
 __constant__ Places kPlaces = places();
 
 // ------------------------------------------------------------------ the kernel
-
-struct W2Params {
-    int W, H, F, r, T, rgb, tiles_x;
-    int tw, gx, gy;          // pixel group tw x (16 / tw), groups across and down
-    int part;                // neighbour pairs per partial sum
-    int flush;               // some window has more pairs than that
-    int seg;                 // neighbour pairs per table
-    float h, log_eps, ridge;
-    const float* radiance;   // [F][C][H][W]
-    const float* features;   // [F][7][H][W]
-    const float* bandwidth;  // [7]
-    float4* packed;          // [F][2][H][W]: (y, normal xyz), (depth, albedo rgb)
-    float* alpha;            // [F][H][W]
-};
 
 // Dynamic shared memory.  Accumulation: flushed sums [sum][warp][pixel], table
 // [pair][entry][lane]; solve: the matrix, over both.
@@ -638,6 +610,16 @@ int part_pairs(int pairs)
     return kPart;
 }
 
+// Inputs of at most this many pixel groups take the Gram kernel (wlr2_gram.cu, with
+// both sides measured); ESIM_AD_WLR2_SMALL overrides the line.
+unsigned long long small_groups()
+{
+    if (const char* e = getenv("ESIM_AD_WLR2_SMALL")) {
+        if (*e) return strtoull(e, nullptr, 10);
+    }
+    return 64;
+}
+
 }  // namespace
 }  // namespace esim
 
@@ -680,6 +662,7 @@ extern "C" esim_ad_status esim_ad_wlr2_forward(const esim_ad_wlr_desc* d, const 
     p.gy = (p.H + kPix / p.tw - 1) / (kPix / p.tw);
     const unsigned long long n = groups(p.tw) * (unsigned long long)p.F;
     if (n > 0x7fffffffull) return ESIM_AD_EINVAL;
+    const bool small = n <= small_groups();
     const int S = 2 * d->radius + 1;
     const int pairs = (S * S + 1) / 2 * (d->frames < d->sequence ? d->frames : d->sequence);
     p.part = part_pairs(pairs);
@@ -691,6 +674,10 @@ extern "C" esim_ad_status esim_ad_wlr2_forward(const esim_ad_wlr_desc* d, const 
     const dim3 pack_grid(p.tiles_x * ((d->height + kTileY - 1) / kTileY), d->sequence);
     wlr2_pack_kernel<<<pack_grid, kTilePix, 0, s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return ESIM_AD_ECUDA;
+    if (small) {
+        const cudaError_t e = launch_wlr2_gram(p, s);
+        return e == cudaSuccess ? ESIM_AD_OK : e == cudaErrorInvalidValue ? ESIM_AD_EINVAL : ESIM_AD_ECUDA;
+    }
     if (cudaFuncSetAttribute(wlr2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMatBytes) != cudaSuccess)
         return ESIM_AD_ECUDA;
     wlr2_kernel<<<(unsigned)n, kThreads, kMatBytes, s>>>(p);

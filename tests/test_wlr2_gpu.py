@@ -117,3 +117,31 @@ def test_wlr2_deterministic_and_validates():
         wlr2(rad.cuda(), feat.cuda(), radius=0)
     with pytest.raises((EsimError, ValueError)):
         wlr2(rad.cuda(), feat.cuda(), radius=3, frames=17)
+
+
+@pytest.mark.parametrize("W,H,F,r,T", [
+    (1, 1, 1, 1, 1),
+    (16, 1, 1, 3, 1),
+    (17, 2, 2, 2, 2),
+    (8, 4, 1, 3, 1),
+    (9, 5, 1, 3, 1),
+    (12, 9, 3, 5, 3),
+    (20, 17, 2, 12, 2),
+])
+def test_wlr2_moments_of_small_inputs(W, H, F, r, T, monkeypatch):
+    """The edges of the kernel for larger inputs, at sizes that it leaves to the other one."""
+    monkeypatch.setenv("ESIM_AD_WLR2_SMALL", "0")
+    test_wlr2_pixel_groups_and_partial_sums(W, H, F, r, T)
+
+
+@pytest.mark.parametrize("W,H,F,gram", [(24, 20, 2, True), (16, 64, 1, True), (16, 65, 1, False), (41, 29, 1, False)])
+def test_wlr2_kernel_by_the_number_of_pixel_groups(W, H, F, gram, monkeypatch):
+    """Up to 64 groups of 16 pixels take the Gram kernel; the two kernels round differently."""
+    rad, feat = _inputs(W, H, F, True, seed=2)
+    chosen = _gpu(rad, feat, radius=3, frames=2)
+    by_line = {}
+    for line in ("0", "1000000"):
+        monkeypatch.setenv("ESIM_AD_WLR2_SMALL", line)
+        by_line[line] = _gpu(rad, feat, radius=3, frames=2)
+    assert not np.array_equal(by_line["0"], by_line["1000000"])
+    assert np.array_equal(chosen, by_line["1000000" if gram else "0"])
