@@ -128,22 +128,23 @@ __device__ __forceinline__ float hit_sphere(float4 oc, V3 d, float eps)
     return t > eps ? t : fa(-b, sq);
 }
 
-// The wall (or the open front) a ray from inside the room reaches.
+// The wall (or the open front) a ray from inside the room reaches; a direction
+// that is not a number reaches none.
 __device__ __forceinline__ Hit hit_walls(const esim_ad_render_scene& sc, V3 o, V3 d)
 {
     Hit h{INFINITY, 5};
     const float tx = fd(fs(d.x > 0.0f ? sc.box[0] : -sc.box[0], o.x), d.x);
-    if (d.x != 0.0f) {
+    if (fabsf(d.x) > 0.0f) {
         h.t = tx;
         h.kind = d.x > 0.0f ? 1 : 0;
     }
     const float ty = fd(fs(d.y > 0.0f ? sc.box[1] : -sc.box[1], o.y), d.y);
-    if (d.y != 0.0f && ty < h.t) {
+    if (fabsf(d.y) > 0.0f && ty < h.t) {
         h.t = ty;
         h.kind = d.y > 0.0f ? 3 : 2;
     }
     const float tz = fd(fs(d.z > 0.0f ? sc.box[2] : -sc.box[2], o.z), d.z);
-    if (d.z != 0.0f && tz < h.t) {
+    if (fabsf(d.z) > 0.0f && tz < h.t) {
         h.t = tz;
         h.kind = d.z > 0.0f ? 5 : 4;
     }

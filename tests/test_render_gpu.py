@@ -121,3 +121,19 @@ def test_gpu_second_interaction_only_adds_light():
     r1 = _np(render(cornell(width=40, height=30, spp=2, max_bounces=1), 2))["radiance"]
     r2 = _np(render(cornell(width=40, height=30, spp=2, max_bounces=2), 2))["radiance"]
     assert np.all(r2 >= r1) and (r2 > r1).mean() > 0.5
+
+
+@pytest.mark.parametrize("n_spheres", [0, 3])
+def test_rays_without_a_direction_see_nothing(n_spheres):
+    """An infinite field of view leaves every camera ray without a direction: it
+    leaves through the open front, and the frame is black."""
+    import paper_2303_02608_gb300 as m
+    from types import SimpleNamespace
+    spheres = [SimpleNamespace(center=(0.2 * j, -0.5, -0.5), velocity=(0.0, 0.0, 0.0), radius=0.1,
+                               albedo=(0.5, 0.5, 0.5)) for j in range(n_spheres)]
+    scene = SimpleNamespace(width=24, height=16, spp=2, max_bounces=2, seed=3, cam_pos=(0.0, 0.0, 1.4),
+                            tan_half_fov_y=float("inf"), box=(1.0, 1.0, 1.5), wall_albedo=((0.7, 0.7, 0.7),) * 5,
+                            back_albedo2=(0.2, 0.2, 0.25), checker=0.25, light=(-0.3, 0.3, -0.6, 0.0),
+                            light_radiance=(17.0, 12.0, 4.0), eps=1e-4, spheres=spheres)
+    for name, v in m.render(scene, 0).items():
+        assert not v.any(), name
