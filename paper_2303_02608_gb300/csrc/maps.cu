@@ -38,8 +38,26 @@ __global__ void __launch_bounds__(kMapThreads) copy_maps_kernel(const float* alp
     }
 }
 
-// Memory of this device that 16-byte accesses can reach.
-bool reachable(const void* p, int device)
+typedef CUresult (*AddressRangeFn)(CUdeviceptr*, size_t*, CUdeviceptr);
+
+AddressRangeFn address_range_fn()
+{
+    static const AddressRangeFn fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<AddressRangeFn>(f);
+    }();
+    return fn;
+}
+
+// Memory of this device that 16-byte accesses can reach, `bytes` of it within one
+// allocation (a copy call checks that; the kernel would write past it).
+bool reachable(const void* p, size_t bytes, int device)
 {
     if (reinterpret_cast<uintptr_t>(p) & 15u) return false;
     cudaPointerAttributes a;
@@ -47,7 +65,12 @@ bool reachable(const void* p, int device)
         cudaGetLastError();
         return false;
     }
-    return a.type == cudaMemoryTypeDevice && a.device == device;
+    if (a.type != cudaMemoryTypeDevice || a.device != device) return false;
+    const AddressRangeFn range = address_range_fn();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    return range && range(&base, &size, at) == CUDA_SUCCESS && at - base <= size && size - (at - base) >= bytes;
 }
 
 }  // namespace
@@ -56,12 +79,13 @@ cudaError_t copy_maps(const float* alpha, float* alpha_out, const uint8_t* flag,
                       bool to_device, int device, cudaStream_t s)
 {
     if (!alpha_out && !flag_out) return cudaSuccess;
-    if (to_device && (!alpha_out || reachable(alpha_out, device)) && (!flag_out || reachable(flag_out, device))) {
+    if (to_device && (!alpha_out || reachable(alpha_out, n * sizeof(float), device)) &&
+        (!flag_out || reachable(flag_out, n, device))) {
         const size_t blocks = (n + 16 * kMapThreads - 1) / (16 * kMapThreads);
         copy_maps_kernel<<<(unsigned)blocks, kMapThreads, 0, s>>>(alpha, alpha_out, flag, flag_out, n);
         return cudaGetLastError();
     }
-    // host buffers, another device's, or unaligned ones
+    // host buffers, another device's, unaligned ones, or ones that are too small (refused)
     const cudaMemcpyKind k = to_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     cudaError_t e = alpha_out ? cudaMemcpyAsync(alpha_out, alpha, n * sizeof(float), k, s) : cudaSuccess;
     if (e == cudaSuccess && flag_out) e = cudaMemcpyAsync(flag_out, flag, n, k, s);

@@ -36,3 +36,29 @@ def test_denoised_into_any_buffer(W, H):
                 exp_f[off:off + n] = host_f
             assert torch.equal(buf_a.cpu(), exp_a) and torch.equal(buf_f.cpu(), exp_f)
     sim.close()
+
+
+@pytest.mark.parametrize("alpha_bytes,flag_bytes", [(256, 1 << 20), (1 << 20, 256)])
+def test_denoised_into_a_buffer_that_is_too_small(alpha_bytes, flag_bytes):
+    """An allocation smaller than its map is refused, as a copy call refuses it."""
+    import ctypes
+    import paper_2303_02608_gb300 as m
+    W, H = 64, 65
+    sim = m.Simulator(m.SimConfig(width=W, height=H, radius=2, frames=2, contrast=0.1, rgb=True))
+    f = Scene(SceneConfig(kind="rects", width=W, height=H, frames=1, spp=2, seed=2, rgb=True, n_rects=3)).sequence()[0]
+    sim.push({k: f[k].cuda() for k in ("radiance", "normal", "albedo", "depth")})
+    cu = ctypes.CDLL("libcuda.so.1")
+    ptrs = []
+    for size in (alpha_bytes, 1 << 18, flag_bytes, 1 << 18):   # with room of our own behind each
+        p = ctypes.c_uint64()
+        assert cu.cuMemAlloc_v2(ctypes.byref(p), ctypes.c_size_t(size)) == 0
+        ptrs.append(p.value)
+    try:
+        with pytest.raises(m.EsimError) as e:
+            m.esim_ad_denoised(sim.ctx, ptrs[0], ptrs[2], True)
+        assert e.value.status == m.ESIM_AD_ECUDA
+    finally:
+        sim.close()
+        torch.cuda.synchronize()
+        for p in ptrs:
+            cu.cuMemFree_v2(ctypes.c_uint64(p))
