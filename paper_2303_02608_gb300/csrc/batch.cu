@@ -375,6 +375,7 @@ WlrParams global_wlr(const esim_ad_batch* b)
     }
     p.ridge = c0.ridge;
     p.sparse_stage = 1;
+    p.box_rows = kRowsSmall;   // the tile's height may change from step to step
     p.poll_limit = kPollLimit;
     p.withhold_copy = 0;
     p.flag_list = b->flag_list;
@@ -654,7 +655,7 @@ esim_ad_status esim_ad_batch_init(const esim_ad_config* cfgs, int32_t n_seq, voi
     {
         std::vector<RingMaps> maps(n_seq);
         for (int i = 0; i < n_seq; ++i)
-            if (!encode_boxes(&maps[i], b->ring[i], cfgs[i].width, cfgs[i].height, c0.frames, b->mixed))
+            if (!encode_boxes(&maps[i], b->ring[i], cfgs[i].width, cfgs[i].height, c0.frames, b->mixed, kRowsSmall))
                 return fail(ESIM_AD_ECUDA);
         if (cudaMemcpy(b->d_maps, maps.data(), sizeof(RingMaps) * n_seq, cudaMemcpyHostToDevice) != cudaSuccess)
             return fail(ESIM_AD_ECUDA);

@@ -48,13 +48,13 @@ bool encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t rank, const
 
 // The ring as rows of 16-byte records, so that a box's rows are contiguous runs:
 // mixed form {8W halves, H, T}, FP32 form {4W floats, H, 2T half-planes}.
-bool encode_boxes(RingMaps* m, const void* ring, int W, int H, int T, bool mixed)
+bool encode_boxes(RingMaps* m, const void* ring, int W, int H, int T, bool mixed, int rows)
 {
     const cuuint32_t el = mixed ? 8 : 4;
     const CUtensorMapDataType dt = mixed ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const cuuint64_t dims[3] = {(cuuint64_t)el * W, (cuuint64_t)H, (cuuint64_t)((mixed ? 1 : 2) * T)};
     const cuuint64_t strides[2] = {(cuuint64_t)16 * W, (cuuint64_t)16 * W * H};
-    const cuuint32_t small[3] = {el * kPitchSmall, (cuuint32_t)kRowsSmall, mixed ? 1u : 2u};
+    const cuuint32_t small[3] = {el * kPitchSmall, (cuuint32_t)rows, 1u};
     const cuuint32_t large[3] = {el * kPitchLarge, (cuuint32_t)kRowsLarge, 1u};
     return encode_tiled(&m->box_small, dt, 3, ring, dims, strides, small) &&
            (!mixed || encode_tiled(&m->box_large, dt, 3, ring, dims, strides, large));
@@ -307,7 +307,8 @@ esim_ad_status encode_ring_map(esim_ad_ctx* c)
     const int rows = wlr_rows(c->cfg.radius, mixed);
     if (rows && !encode(&c->maps.rows, kTileX, rows)) return ESIM_AD_ECUDA;
     return encode(&c->maps.tile, kTileX, kTileY) && encode(&c->maps.ex_tile, kExTileX, kExTileY) &&
-                   encode_boxes(&c->maps, c->ring, c->W, c->H, c->cfg.frames, mixed)
+                   encode_boxes(&c->maps, c->ring, c->W, c->H, c->cfg.frames, mixed,
+                                small_box_rows(c->cfg.radius, kTileY))
                ? ESIM_AD_OK
                : ESIM_AD_ECUDA;
 }
@@ -715,6 +716,7 @@ esim_ad_status esim_ad_push_frame(esim_ad_ctx* c, const esim_ad_frame* fin)
     wp.sparse_max = c->sparse_max;
     wp.rows_min = c->rows_min;
     wp.flag_list = c->flag_list;
+    wp.box_rows = small_box_rows(c->cfg.radius, kTileY);
     wp.sparse_stage = c->sparse_stage;
     wp.tile_base = c->tile_base;
     wp.gram = c->gram;

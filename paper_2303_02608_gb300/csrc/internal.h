@@ -170,6 +170,7 @@ struct WlrParams {
     uint32_t rows_min;               // queue mode: from this many flagged pixels on -> row boxes
     uint32_t sparse_max;             // queue mode: at most this many flagged pixels -> sparse kernel
     const uint32_t* flag_list;       // flagged pixel indices per tile, each run padded to 4 entries
+    int box_rows;                    // rows of a small window box
     int sparse_stage;                // sparse kernel: 1 stage window boxes in shared memory, 0 read via L1
     const uint32_t* tile_base;       // position of each queued tile's run in flag_list
     float* gram;                     // Gram records [entries][68]: entry = pixel index (dense) or
@@ -230,8 +231,8 @@ struct RingMaps {
 // Tiled map without swizzle or interleave; out-of-range elements read as zero.
 bool encode_tiled(CUtensorMap* m, CUtensorMapDataType dt, cuuint32_t rank, const void* ptr, const cuuint64_t* dims,
                   const cuuint64_t* strides, const cuuint32_t* box);
-// The window boxes of a ring (box_large stays as it is in the FP32 form).
-bool encode_boxes(RingMaps* m, const void* ring, int W, int H, int T, bool mixed);
+// The window boxes of a ring, small ones of `rows` rows (box_large stays as it is in the FP32 form).
+bool encode_boxes(RingMaps* m, const void* ring, int W, int H, int T, bool mixed, int rows);
 // Regression pass 1: dense frames (every tile) and adaptive frames (one launch
 // choosing on the device between the sparse window-box form and the
 // tile-staged queue form); the adaptive kernel's shared memory is the larger

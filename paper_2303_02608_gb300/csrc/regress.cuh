@@ -15,7 +15,7 @@ namespace {
 struct SeqView {
     int W, H, t, T, n_tau;
     const void* ring;
-    const CUtensorMap* box_small;   // the ring in boxes of kPitchSmall x kRowsSmall records
+    const CUtensorMap* box_small;   // the ring in boxes of kPitchSmall x box_rows records (FP32: of one half-plane)
     const CUtensorMap* box_large;   // mixed form: kPitchLarge x kRowsLarge
 };
 
@@ -208,15 +208,20 @@ __device__ __noinline__ void refine_fp64(const WlrParams& p, uint32_t pix, const
 // edge), 8 lanes per pixel (16 or 32 when the item holds only two or one
 // pixel, the tail of a tile's run).  For each frame of the temporal window the
 // bounding box of the four windows (clipped to the image) is copied from the
-// ring into the warp's shared memory by one TMA box load, completing on the
-// warp's mbarrier: a box of fixed size from the windows' first corner, the ring
-// seen as rows of records (what lies past the image reads as zero, and no
-// window reaches it).  Boxes of up to 20 x 20 records are double-buffered: frame
-// k+1's copy is issued before frame k is summed.  Larger boxes take the whole
-// buffer one frame at a time; boxes too large for it are read through L1.
-// BOXMEASURED  The lanes split each window's
-// offsets and accumulate the 65 sums in packed FP32 pairs; the g lanes of a
-// pixel are then reduced by shuffles and store one Gram record at the pixel's
+// ring into the warp's shared memory by a TMA box load (FP32: one per half-plane),
+// completing on the warp's mbarrier: a box of fixed size from the windows' first
+// corner, the ring seen as rows of records (what lies past the image reads as zero,
+// and no window reaches it).  Boxes of up to 20 x 20 records are double-buffered in
+// the precision form: frame k+1's copy is issued before frame k is summed.  Their
+// height is what the windows of one tile's pixels can take (box_rows): whole
+// boxes of 20 rows made small FP32 windows slower than copying only their rows.
+// Larger boxes take the whole buffer one frame at a time; boxes too large for it
+// are read through L1.  Pass 1 in us, a bulk copy per window row -> boxes, 1920 x 1080:
+// 15 x 15 x 5 window, 20,800 flagged pixels spread evenly 134 -> 124 (FP32 161 -> 133),
+// 27,100 along edges 139 -> 132 (145 -> 130); 3 x 3 x 3, 41,700 spread 51.9 -> 50.6 (83.8 ->
+// 78.7, with 20 rows 89.1).  The lanes split each window's offsets and accumulate
+// the 65 sums in packed FP32 pairs; the g lanes of a pixel are then added through the
+// warp's buffer (store_records) into one Gram record at the pixel's
 // position in the flagged list.  Warps fetch work independently; there is no
 // block barrier inside the loop, and every mbarrier wait is bounded.
 template <int kItem, bool kMixed, class Src>
@@ -371,12 +376,14 @@ __device__ __forceinline__ void sparse_body(const WlrParams& p, const Src& src)
             if (lane == 0) {
                 const int slot = (sv.t - k) % sv.T;
                 unsigned char* dst = wbuf + (mode == 2 ? b * (kBoxBytes / 2) : 0);
+                const uint32_t small = (uint32_t)(16 * kPitchSmall * p.box_rows);
                 if (kMixed) {
-                    mbar_arrive_expect_tx(&bar[b], mode == 2 ? (uint32_t)kBoxBytes / 2u : (uint32_t)kBoxBytes);
+                    mbar_arrive_expect_tx(&bar[b], mode == 2 ? small : (uint32_t)kBoxBytes);
                     tma_load_3d(dst, mode == 2 ? sv.box_small : sv.box_large, &bar[b], 8 * bx0, by0, slot);
                 } else {
-                    mbar_arrive_expect_tx(&bar[b], (uint32_t)kBoxBytes);
+                    mbar_arrive_expect_tx(&bar[b], 2u * small);
                     tma_load_3d(dst, sv.box_small, &bar[b], 4 * bx0, by0, 2 * slot);
+                    tma_load_3d(dst + kBoxBytes / 2, sv.box_small, &bar[b], 4 * bx0, by0, 2 * slot + 1);
                 }
             }
         };

@@ -24,6 +24,12 @@ constexpr int kBoxWarps = kTilePix / 32;
 static_assert(kPitchSmall * kRowsSmall * 32 == kBoxBytes && kPitchLarge * kRowsLarge * 16 == kBoxBytes,
               "boxes fill the buffer or its halves; an FP32 box's second half-plane starts at the middle");
 
+// Rows of a small box for pixels that share a tile of tile_h rows.
+__host__ __device__ constexpr int small_box_rows(int r, int tile_h)
+{
+    return 2 * r + tile_h < kRowsSmall ? 2 * r + tile_h : kRowsSmall;
+}
+
 struct BoxLayout {
     int tab_small, tab_large, bar_off, buf_off, total;
 };
