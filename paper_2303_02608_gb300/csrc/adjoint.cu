@@ -137,11 +137,11 @@ __device__ __forceinline__ void solve_theta_v(Acc& a, const float (&s2)[NZ], flo
     }
 }
 
-// Sums of the normal equations in packed FP32 pairs, every sum in the order of
-// accum_core (a packed FMA rounds each half as a single one does), regressors
-// in pairs U_k = (u_2k, u_2k+1), u_0 = 1: column j of the Gram's triangle from
-// row 2k on is w U_k * u_j, and what is left over are the diagonal entries of
-// odd rows.
+// Sums of the normal equations in packed FP32 pairs (a packed FMA rounds each half
+// as a single one does), regressors in pairs U_k = (u_2k, u_2k+1), u_0 = 1.  Per
+// neighbour w U_k is rounded first, then multiplied into the running sums: column
+// j of the Gram's triangle from row 2k on takes (w U_k) * u_j, and what is left over
+// are the diagonal entries of odd rows.
 struct FwdSums {
     float2 g[25];   // column 0: rows 0-9; columns 1, 2: rows 2-9; 3, 4: rows 4-9; 5, 6: rows 6-9; 7, 8: rows 8, 9
     float d[5];     // rows and columns 1, 3, 5, 7, 9

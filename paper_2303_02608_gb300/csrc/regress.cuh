@@ -328,7 +328,6 @@ __device__ __forceinline__ void sparse_body(const WlrParams& p, const Src& src)
         const uint32_t pix_e = __shfl_sync(0xffffffffu, e4, split ? part : grp);
         const bool active = grp < m;
         const uint32_t pix = active ? src.pixel(pix_e) : 0u;
-        const uint32_t entry = base + (uint32_t)(split ? part : grp);
         const int cx = (int)(pix % (uint32_t)sv.W), cy = (int)(pix / (uint32_t)sv.W);
         const int dxlo = max(-p.r, -cx), dxhi = min(p.r, sv.W - 1 - cx);
         const int dylo = max(-p.r, -cy), dyhi = min(p.r, sv.H - 1 - cy);

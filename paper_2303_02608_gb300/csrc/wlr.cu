@@ -47,10 +47,6 @@
 
 namespace esim {
 
-namespace {
-
-}  // namespace
-
 // Per-stage metadata published by the producer thread with each staged frame.
 struct StageInfo {
     int tile;   // tile index, or -1: no more work (end of the CTA's stream)

@@ -550,7 +550,8 @@ __global__ void __launch_bounds__(kThreads, 2) wlr2_kernel(const W2Params p)
             __syncwarp();
 #pragma unroll
             for (int i = 0; i < kB; ++i) {
-                // 1 / sqrt of the pivot: one Newton step on the approximation
+                // 1 / sqrt of the pivot: one Newton step on the approximation, within 0.62 units in
+                // the last place (a rounded root and division: 0.75)
                 const float piv = fmaxf(g[diag_elem(i, i)], 1e-30f), r0 = rsqrtf(piv);
                 const float inv = fmaf(0.5f * r0, fmaf(-piv * r0, r0, 1.0f), r0);
 #pragma unroll

@@ -22,46 +22,6 @@ struct Acc {
     float B[NZ];
 };
 
-// One neighbour with log brightness y and seven feature values f (raw
-// features, or the stored values of the mixed form); sc[j] turns a feature
-// difference into its regressor, cf[j] = sc[j] * f_centre[j].
-__device__ __forceinline__ void accum_core(Acc& a, float y, float f0, float f1, float f2, float f3,
-                                           float f4, float f5, float f6, float u1, float u2,
-                                           float en0, const float* __restrict__ sc,
-                                           const float (&cf)[7])
-{
-    float u[NZ];
-    u[0] = 1.0f;
-    u[1] = u1;
-    u[2] = u2;
-    u[3] = fmaf(f0, sc[0], -cf[0]);
-    u[4] = fmaf(f1, sc[1], -cf[1]);
-    u[5] = fmaf(f2, sc[2], -cf[2]);
-    u[6] = fmaf(f3, sc[3], -cf[3]);
-    u[7] = fmaf(f4, sc[4], -cf[4]);
-    u[8] = fmaf(f5, sc[5], -cf[5]);
-    u[9] = fmaf(f6, sc[6], -cf[6]);
-    float en = en0;  // -(u1^2 + u2^2)
-#pragma unroll
-    for (int j = 3; j < NZ; ++j) en = fmaf(-u[j], u[j], en);
-    const float w = ex2_approx(en);
-    const float wy = w * y;
-    float wu[NZ];
-    wu[0] = w;
-#pragma unroll
-    for (int j = 1; j < NZ; ++j) wu[j] = w * u[j];
-    a.G[0] += w;
-#pragma unroll
-    for (int i = 1; i < NZ; ++i) {
-        a.G[tri(i, 0)] += wu[i];
-#pragma unroll
-        for (int j = 1; j <= i; ++j) a.G[tri(i, j)] = fmaf(wu[i], u[j], a.G[tri(i, j)]);
-    }
-    a.B[0] += wy;
-#pragma unroll
-    for (int i = 1; i < NZ; ++i) a.B[i] = fmaf(wy, u[i], a.B[i]);
-}
-
 // ---------------------------------------------------------------------------
 // Packed accumulation.  The 65 sums of the normal equations (the 55 entries of
 // the Gram matrix of z = (1, u) and the 10 of the right-hand side) are held as
@@ -392,23 +352,6 @@ __device__ __forceinline__ void gram_load(const float* __restrict__ rec, Acc& a)
         else if (j == 10) a.B[i] = v[s];
         else a.G[i >= j ? tri(i, j) : tri(j, i)] = v[s];
     }
-}
-
-// FP32 ring: h0 = (y, normal xyz), h1 = (depth, albedo rgb).
-__device__ __forceinline__ void accumulate(Acc& a, const float4 h0, const float4 h1, float u1,
-                                           float u2, float en0, const float* __restrict__ sf,
-                                           const float (&cf)[7])
-{
-    accum_core(a, h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w, u1, u2, en0, sf, cf);
-}
-
-// Mixed ring: one 16-byte record (FP16 y, BF16 stored features).
-__device__ __forceinline__ void accumulate(Acc& a, const uint4 v, float u1, float u2, float en0,
-                                           const float* __restrict__ qs, const float (&cf)[7])
-{
-    float y, q[7];
-    unpack_mixed(v, y, q);
-    accum_core(a, y, q[0], q[1], q[2], q[3], q[4], q[5], q[6], u1, u2, en0, qs, cf);
 }
 
 // Ridge, Jacobi equilibration and Cholesky solve of the packed 10x10 system.
