@@ -228,8 +228,7 @@ __device__ __forceinline__ float nearest2(const QualParams& p, int s, int pol, i
 #pragma unroll
                 for (int i = 0; i < kStep; ++i) {
                     const float dx = (float)(j0 + i) * p.invW;
-                    const G m = min(l[i], r[i]);
-                    const float dy = m == kNoEvent<G> ? INFINITY : (float)m * p.invH;
+                    const float dy = (float)min(l[i], r[i]) * p.invH;
                     // dy^2 is rounded by itself: contracted into the sum, distances that equal
                     // a threshold would fall on its other side
                     best = fminf(best, __fadd_rn(fmaf(dx, dx, dt2), __fmul_rn(dy, dy)));
@@ -237,7 +236,9 @@ __device__ __forceinline__ float nearest2(const QualParams& p, int s, int pol, i
             }
         }
     }
-    return best;
+    // Two events are less than sqrt(3) apart; rows that stand for "no event" give at least 4
+    // (2^32 - 1 rows of at most 2^31, 2^16 - 1 of at most 4096).
+    return best < 3.5f ? best : INFINITY;
 }
 
 // 4096 pixels of the query set per block; blockIdx.y = direction (0: generated
