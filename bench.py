@@ -558,9 +558,9 @@ def _paper_density(args, dev, stream, fp32_peak, sink):
         out[name] = {"value": round(N * K / (ms * 1e-3), 1), "unit": UNIT, "ms_per_step": round(ms / K, 4),
                      "flagged_fraction": round(phi, 4), "events_per_step": round(ev / K, 1),
                      "kernel_ms_per_step": {k: round(v / K, 4) for k, v in prof["ms"].items()},
-                     "regression_kernel": ("dense tile-staged (every pixel)" if mode == ESIM_AD_EXHAUSTIVE else
-                                           "tile-staged over the flagged-tile queue when more than 1/8 of the "
-                                           "pixels are flagged, else per-warp window boxes"),
+                     "regression_kernel": ("every pixel" if mode == ESIM_AD_EXHAUSTIVE else
+                                           "the flagged-tile queue, by row boxes or tile-staged, when more than 1/8 "
+                                           "of the pixels are flagged, else per-warp window boxes"),
                      "regression_roofline": {"achieved": round(ach, 3), "frac": round(ach / fp32_peak, 4),
                                              "frac_at_145": round(ach / fp32_peak * 145 / FLOP_PER_NEIGHBOUR, 4),
                                              "launch_ms": round(wlr_ms / n_launch, 4)}}

@@ -10,10 +10,11 @@
 // Of a warp's lanes each quarter reads 8 neighbouring records: no bank
 // conflicts.  Offsets outside the image get weight 0 through their distance
 // (the copy fills them with zeros); those outside for every pixel are left out
-// (a frame of 17 x 5, 21 x 21 x 4 window: 107 us, 130 with them, 125 tile-staged).  While a tile's sums are reduced and stored
-// the next tile's frames land; the other CTA of the SM covers the rest.
+// (a frame of 17 x 5, 21 x 21 x 4 window: 107 us, 130 with them, 125 tile-staged).
+// While a tile's sums are reduced and stored the next tile's frames land; the
+// other CTA of the SM covers the rest.
 //
-// It takes the windows where it wins at every image size: radius 7 and up, at
+// It takes the windows where it wins at the image sizes measured: radius 7 and up, at
 // least 4 frames (5 in the FP32 form, whose records cost no unpacking that the
 // factored sums could share), and all frames of a tile fitting together.  Fewer
 // frames or offsets do not repay the work per offset and the four lanes' sum.
@@ -22,10 +23,15 @@
 // -> 4494 / 174; FP32, 5 frames 5216 / 219 -> 5152 / 197.  Not taken: FP32, 4 frames
 // 4215 / 191 -> 4415 / 174; radius 5, 4 frames, precision form 2567 / 141 -> 2612 /
 // 122; with frames in two groups (FP32, radius 9, 5 frames) 900 x 700 3613 -> 4109.
+// Whole frames of the other windows that fit, tile-staged / here, 16 windows
+// (precision form: radius 7 with 4 to 12 frames, 8 and 9 with 4 and 5, 10 to 13 with 4;
+// FP32: radius 7 with 5 and 6, 8 with 5): 1500 x 1000 1.01-1.13, 640 x 480 1.01-1.16, 333 x 251
+// 1.28-1.47, 200 x 150 1.07-1.21, 64 x 48 2.0-2.9.  Only images of a few pixels lose, by
+// the window's part that reaches no pixel: 5 x 17, 27 x 27 x 4 window 132 us for 124.
 // The choice does not look at the image's size: a pixel's sums are rounded the
 // same way in any image or strip.
 //
-// FP32-bound, 70% of the FMA pipe.  1920 x 1080, 15 x 15 x 5 window, precision
+// FP32-bound: the FMA pipe is 70% busy (960 x 540).  1920 x 1080, 15 x 15 x 5 window, precision
 // form: a frame takes 7.32 ms, 7.65 with the tile-staged kernel (the frames'
 // loop not unrolled costs 3% more, its first frame peeled 8%).  Its alpha is also
 // nearer to float64 (3e-7 against 2e-6, relative).

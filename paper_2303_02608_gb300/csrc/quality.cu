@@ -251,6 +251,9 @@ __device__ __forceinline__ float nearest2(const QualParams& p, int s, int pol, i
 // 7.35 ms with a thread per pixel, 3.27 with lists of 2048 pixels, 1.80 with
 // slots in place of atomics and 1024 pixels, 1.24 with 4096 pixels and eight
 // columns a step (1024 pixels: partly filled warps; 64 or 256 threads: slower).
+// Small and dense sets gain too (whole evaluations, a thread per pixel -> here): 96 x
+// 64 x 6 with 1% and all of the pixels 109 -> 87 and 124 -> 121 us, 160 x 120 x 10 135 -> 93 and
+// 219 -> 124, 1280 x 720 x 30 2.4 -> 0.32 and 11.4 -> 1.03 ms.
 template <class G>
 __global__ void __launch_bounds__(kQueryThreads) query_kernel(QualParams p)
 {

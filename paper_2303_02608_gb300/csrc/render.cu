@@ -15,8 +15,8 @@
 // whatever its signs; the offsets from a hit point to the spheres serve both
 // its shadow ray and the bounce that leaves it; a shadow ray stops at its first
 // blocker.  All of it with the same operations on the same values.  1920 x 1080,
-// 4 samples, two interactions: 315 us with three spheres (336 before; 227 / 247
-// with none, 466 / 535 with eight).  Keeping the spheres' offsets takes
+// 4 samples, two interactions: 301 us with three spheres (336 before), 224 / 244
+// with none, 457 / 523 with eight.  Keeping the spheres' offsets takes
 // registers: four CTAs per SM up to four spheres, three beyond, measured faster
 // than what the compiler chooses (354 us at two per SM).
 // Random numbers: Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11), key

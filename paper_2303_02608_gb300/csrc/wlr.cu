@@ -403,12 +403,13 @@ __device__ __forceinline__ void tile_body(const CUtensorMap& tmap, const WlrPara
 // rarely need more rows than a box holds; those that do are done in passes.
 // Four warps per scheduler hide the wait for a copy (1-2 us against the 30-40
 // of summing a frame).  FP32-bound: 1920 x 1080, 500,000 pixels flagged, 15 x 15 x 5
-// window, precision form: 2121 us (53% of the FP32 peak), tile-staged 2543.
-// Taken when work items are whole tiles (rows_min, the total from which
-// queue_chunk gives 256).  Below that an item has many lanes per pixel and little
-// to sum per frame, and a warp's one box in flight shows: frames of 480 x 300, 7 x 7 x 3
-// window, took 195 us against 153 tile-staged, 15 x 15 x 5 327 against 308; of
-// 1500 x 1000, above it, 404 against 457 and 1623 against 1924.
+// window, precision form: 2121 us (53% of the FP32 peak by the method's operations,
+// the FMA pipe 73% busy), tile-staged 2543.  Taken when work items are whole tiles
+// (rows_min, the total from which queue_chunk gives 256).  Below that an item has
+// many lanes per pixel and little to sum per frame, and a warp's one box in flight
+// shows: frames of 480 x 300, 7 x 7 x 3 window, took 195 us against 153 tile-staged,
+// 15 x 15 x 5 327 against 308; of 1500 x 1000, above it, 404 against 457 and 1623 against
+// 1924.
 constexpr int kRowsBytes = 13312;   // per warp; with 8 warps two CTAs fit on an SM
 struct RowsLayout {
     int rows, bar_off, buf_off, total;
